@@ -163,7 +163,10 @@ int mm_set_solver(mm_ctx* ctx, double max_err, double headroom, double dt0,
 int mm_set_fixed_dt_sequence(mm_ctx* ctx, const double* dts, int n);
 
 /* Failure detection (no counterpart in the paper): the row-stage kernels wait
- * for their tensor copies (TMA) on mbarriers, and every such wait is bounded.
+ * for their tensor copies (TMA) on mbarriers, and the film kernel's blocks for
+ * one another at grid barriers; every such wait is bounded (on films whose
+ * rows the stage kernels would not move by tensor copies the limit is always
+ * the default).
  * `cycles` is the limit in SM clock cycles (default 2^30, about half a second
  * at 2.07 GHz); a wait that reaches it records MM_ERR_TIMEOUT in the device
  * state and the attempt is abandoned: the kernel first waits, with the
@@ -313,7 +316,10 @@ int mm_profile_attempts(mm_ctx* ctx, int attempts, int max, int* kinds, double* 
  * axes and, in 3-D, py >= 32 and 16 <= pz <= 64, in 2-D (one layer) py of
  * 128, 256 or 512 (MM_ERR_ARG otherwise).  *active (may be NULL) receives the
  * kernels in use: 1 or 2, or 0 on a grid without the fused layout.  The
- * stepping graph is captured again at the next step. */
+ * stepping graph is captured again at the next step.  Films (one layer of
+ * more than 8 rows, y not periodic) step with a persistent kernel that holds
+ * its own (y, z) part by default; with which = 1 or 2 they step with the
+ * stage kernels. */
 int mm_set_yz_kernels(mm_ctx* ctx, int which, int* active);
 
 /* FP32 fused multiply-add throughput of `device` (no counterpart in the

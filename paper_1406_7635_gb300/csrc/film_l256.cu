@@ -1,0 +1,5 @@
+// The persistent film kernel for x rows of 256 complex values.
+#include "film.cuh"
+
+template bool mm::film_plan_l<256>(const Geom&, int, FilmPlan*);
+template cudaError_t mm::launch_film_l<256>(const FilmPlan&, int, const FilmArgs&, cudaStream_t);

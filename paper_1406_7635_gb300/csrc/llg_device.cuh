@@ -80,23 +80,33 @@ struct FieldParts {
 
 __device__ __forceinline__ float3 f3(float a, float b, float c) { return make_float3(a, b, c); }
 
+// how a kernel reads the material tables: from global memory, or wherever it
+// has staged them
+struct LdGlobal {
+  __device__ __forceinline__ static float at(const float* p) { return __ldg(p); }
+};
+struct LdAny {
+  __device__ __forceinline__ static float at(const float* p) { return *p; }
+};
+
 // uniaxial anisotropy (Ku1 and Ku2 parts) and Zeeman field of region r
+template <class LD = LdGlobal>
 __device__ __forceinline__ void field_local(const RegionLUT* __restrict__ lut, const Terms& T, int r, float3 mi,
                                             float sinft, FieldParts& P) {
   if (T.anis) {
-    const float ux = __ldg(&lut->u[0][r]), uy = __ldg(&lut->u[1][r]), uz = __ldg(&lut->u[2][r]);
+    const float ux = LD::at(&lut->u[0][r]), uy = LD::at(&lut->u[1][r]), uz = LD::at(&lut->u[2][r]);
     const float um = ux * mi.x + uy * mi.y + uz * mi.z;
-    const float a1 = __ldg(&lut->k1[r]) * um;
-    const float a2 = __ldg(&lut->k2[r]) * um * um * um;
+    const float a1 = LD::at(&lut->k1[r]) * um;
+    const float a2 = LD::at(&lut->k2[r]) * um * um * um;
     P.anis1 = f3(a1 * ux, a1 * uy, a1 * uz);
     P.anis2 = f3(a2 * ux, a2 * uy, a2 * uz);
   } else {
     P.anis1 = P.anis2 = f3(0, 0, 0);
   }
   if (T.zeeman) {
-    P.zee = f3(__ldg(&lut->b0[0][r]) + __ldg(&lut->b1[0][r]) * sinft,
-               __ldg(&lut->b0[1][r]) + __ldg(&lut->b1[1][r]) * sinft,
-               __ldg(&lut->b0[2][r]) + __ldg(&lut->b1[2][r]) * sinft);
+    P.zee = f3(LD::at(&lut->b0[0][r]) + LD::at(&lut->b1[0][r]) * sinft,
+               LD::at(&lut->b0[1][r]) + LD::at(&lut->b1[1][r]) * sinft,
+               LD::at(&lut->b0[2][r]) + LD::at(&lut->b1[2][r]) * sinft);
   } else {
     P.zee = f3(0, 0, 0);
   }
@@ -316,8 +326,8 @@ __device__ void check_done(DevState* st) {
 // whose error estimate is of order 2), bounded by dt_max, and
 // at least dt_min after an accepted step; a rejection that would need a step
 // below dt_min ends the call with MM_ERR_DT_UNDERFLOW.
-__device__ void controller_on(DevState* st, StageCoef* sc, double* __restrict__ hist,
-                              const double* __restrict__ fixed) {
+// (hist null: the accepted step size is not recorded)
+__device__ void controller_core(DevState* st, double* __restrict__ hist) {
   const double eps = (double)__uint_as_float(st->err_bits);
   st->err_bits = 0;
   st->ticket = 0;
@@ -344,7 +354,7 @@ __device__ void controller_on(DevState* st, StageCoef* sc, double* __restrict__ 
     st->t += h;
     if (st->mode == 1 && st->t + 1e-6 * h >= st->t_end) st->t = st->t_end;
     st->parity ^= 1;
-    if (st->hist_n < kHistCap) hist[st->hist_n] = h;
+    if (hist && st->hist_n < kHistCap) hist[st->hist_n] = h;
     st->hist_n++;
     st->accepted++;
     if (replay) st->fixed_idx++;
@@ -359,6 +369,12 @@ __device__ void controller_on(DevState* st, StageCoef* sc, double* __restrict__ 
     }
     st->dt = ndt;
   }
+}
+
+// the controller and, unless the call is done, the next attempt's set-up
+__device__ void controller_on(DevState* st, StageCoef* sc, double* __restrict__ hist,
+                              const double* __restrict__ fixed) {
+  controller_core(st, hist);
   if (!st->done) prepare_attempt(st, sc, fixed);
 }
 

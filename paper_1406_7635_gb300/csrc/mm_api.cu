@@ -5,7 +5,8 @@
 // is captured once into a CUDA graph and replayed.  The controller runs on the
 // device and marks the call done; the host only replays the graph and reads the
 // device state back at a few check points, so steps are taken without a
-// host round trip per step.
+// host round trip per step.  Films run whole attempts in one persistent
+// kernel instead (film.cuh): one launch for all steps of a call.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -14,6 +15,7 @@
 #include <vector>
 
 #include "../../include/mm.h"
+#include "film.h"
 #include "mm_internal.h"
 
 using namespace mm;
@@ -78,6 +80,11 @@ struct mm_ctx {
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   SttLUT* stt_lut = nullptr;     // device table
+  // persistent film kernel (film.cuh): its plan (rows = 0: none), second
+  // spectrum buffer and barrier words
+  FilmPlan film;
+  float2* film_spec = nullptr;
+  FilmSync* film_sync = nullptr;
   int method = 0;                // host copy of DevState::method
   bool lut_dirty = true;
   bool m_set = false;
@@ -280,6 +287,66 @@ bool rowstage_path(const mm_ctx* c) {
 // argument: the context keeps the Geom layout unchanged.)
 bool row_dep(const mm_ctx* c) { return c->y2d; }
 
+// Plans the persistent film kernel for the context's grid and makes its
+// buffers fit (at creation and after set_pbc).
+int prepare_film(mm_ctx* c) {
+  if (c->film_spec) cudaFree(c->film_spec);
+  c->film_spec = nullptr;
+  if (!film_plan(c->g, &c->film)) return MM_OK;
+  const size_t bytes = 3 * (size_t)c->g.ny * c->g.hxs * sizeof(float2);
+  MM_CUDA(cudaMalloc((void**)&c->film_spec, bytes));
+  MM_CUDA(cudaMemsetAsync(c->film_spec, 0, bytes, c->stream));
+  if (!c->film_sync) MM_CUDA(cudaMalloc((void**)&c->film_sync, sizeof(FilmSync)));
+  MM_CUDA(cudaMemsetAsync(c->film_sync, 0, sizeof(FilmSync), c->stream));
+  MM_CUDA(cudaStreamSynchronize(c->stream));
+  return MM_OK;
+}
+
+// Whether the context steps with the persistent film kernel: a planned film
+// with the exact demag field and the default (y, z) kernels (a request for
+// particular ones steps with them, in the stage kernels' graph).
+bool film_path(const mm_ctx* c) { return c->film.rows > 0 && c->T.demag && !c->sur_active && c->yz_req == 0; }
+
+// one launch of the film kernel: the first stage alone (k1), or up to
+// `attempts` attempts; begin starts a call of `mode`
+int enqueue_film(mm_ctx* c, bool begin, int mode, long long nsteps, double t_end, bool k1, int attempts) {
+  const Buffers& b = c->b;
+  FilmArgs a{};
+  a.g = c->g;
+  a.T = c->T;
+  a.S = c->stt;
+  a.m0 = b.m[0];
+  a.m1 = b.m[1];
+  for (int j = 0; j < 7; ++j) a.k[j] = b.k[j];
+  a.tw = b.tw;
+  a.kt = b.ktf;
+  a.lut = b.lut;
+  a.xlut = b.xlut;
+  a.code = b.code;
+  a.spec1 = b.spec;
+  a.spec2 = c->film_spec;
+  a.halo = b.ms;
+  a.st = b.st;
+  a.hist = b.hist;
+  a.fixed = b.fixed;
+  a.sync = c->film_sync;
+  a.freq = c->freq;
+  a.phase_over_pi = c->phase / kPi;
+  a.t_end = t_end;
+  a.nsteps = nsteps;
+  a.begin = begin;
+  a.mode = mode;
+  a.k1 = k1;
+  a.attempts = attempts;
+  // (the wait limit applies where the stage kernels' tensor copies would have
+  // been under it, so a film keeps its behaviour at a given limit)
+  a.state_limit = rowstage_path(c) && (c->maps.ok_spec || c->maps.ok_sten);
+  a.oct_sm = c->film.oct_sm;
+  c->launches += 1;
+  MM_CUDA(launch_film(c->film, a, c->stream));
+  return MM_OK;
+}
+
 // stage-1 torque at the current m (FSAL start)
 void enqueue_k1(mm_ctx* c) {
   if (rowstage_path(c)) {
@@ -383,10 +450,34 @@ int status_to_code(int status) {
 // The stepping loop shared by mm_step and mm_run.  Launches are queued
 // without waiting: the begin kernel, the first-stage evaluation and a first
 // batch of attempts; the device state is read back only at check points.
+//
+// Films (film_path): the kernel runs attempts until the call is done, at most
+// kFilmAttempts per launch (a bound on one launch's duration: a fraction of a
+// second on the largest film).
+constexpr int kFilmAttempts = 1024;
+
+int drive_film(mm_ctx* c, int mode, long long nsteps, double t_end) {
+  c->st_fresh = false;
+  const bool k1_was_valid = c->k1_valid;
+  int rc = MM_OK;
+  if (!k1_was_valid) rc = enqueue_film(c, true, mode, nsteps, t_end, true, 1);
+  for (int guard = 0; guard < 1000000 && !rc; ++guard) {
+    rc = enqueue_film(c, guard == 0 && k1_was_valid, mode, nsteps, t_end, false, kFilmAttempts);
+    if (rc) break;
+    rc = read_state(c);
+    if (rc) break;
+    const DevState& s = *c->st_host;
+    c->k1_valid = k1_was_valid || s.call_attempts > 0;
+    if (s.done) return status_to_code(s.status);
+  }
+  return rc ? rc : fail(MM_ERR_STATE, "stepping loop did not finish");
+}
+
 int drive(mm_ctx* c, int mode, long long nsteps, double t_end) {
   if (!c->m_set) return fail(MM_ERR_STATE, "m has not been set");
   int rc = flush_luts(c);
   if (rc) return rc;
+  if (film_path(c)) return drive_film(c, mode, nsteps, t_end);
   rc = build_graph(c);
   if (rc) return rc;
   c->st_fresh = false;   // the stepping kernels write the device state
@@ -594,6 +685,8 @@ int mm_create(mm_ctx** out, int nx, int ny, int nz, double dx, double dy, double
   if (e == cudaSuccess && g.fused) e = prepare_rowstage(g);
   if (e == cudaSuccess) rowstage_maps(g, b, &c->maps);
   if (e != cudaSuccess) return cleanup(fail(MM_ERR_CUDA, std::string("warm-up: ") + cudaGetErrorString(e)));
+  rc = prepare_film(c);
+  if (rc) return cleanup(rc);
   *out = c;
   return MM_OK;
 }
@@ -606,7 +699,7 @@ int mm_destroy(mm_ctx* c) {
   Buffers& b = c->b;
   void* ptrs[] = {b.m[0], b.m[1], b.k[0], b.k[1], b.k[2], b.k[3], b.k[4], b.k[5], b.k[6], b.ms, b.ms2, b.bd, b.out,
                   b.spec, b.kt, b.ktf, b.tw, b.mask, b.region, b.lut, b.xlut, b.code, b.st, b.hist, b.acc,
-                  b.fixed, c->sur_acc, c->stt_lut, c->yzt, b.part};
+                  b.fixed, c->sur_acc, c->stt_lut, c->yzt, b.part, c->film_spec, c->film_sync};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->st_host) cudaFreeHost(c->st_host);
@@ -1001,7 +1094,7 @@ int mm_set_pbc(mm_ctx* c, int px, int py, int pz) {
   if (e != cudaSuccess)
     return fail(e == cudaErrorMemoryAllocation ? MM_ERR_OOM : MM_ERR_CUDA,
                 std::string("set_pbc: ") + cudaGetErrorString(e));
-  return MM_OK;
+  return prepare_film(c);
 }
 
 int mm_get_max_torque(mm_ctx* c, double* tau_max) {
