@@ -18,6 +18,7 @@
 // and the per-mode channel mixing are small complex products on the FP32
 // cores.  Parameters are float32 masters (Adam), used in bfloat16 by the
 // tensor-core products.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -857,8 +858,12 @@ __global__ void k_loss(long long n, const float* __restrict__ yh, const float* _
 
 __global__ void k_dloss(long long n, const float* __restrict__ yh, const float* __restrict__ y,
                         const double* __restrict__ acc, float* __restrict__ dy) {
+  // (one division per block: a float64 division per value was most of this kernel's time)
+  __shared__ double scale;
+  if (threadIdx.x == 0) scale = 2.0 / acc[1];
+  __syncthreads();
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) dy[i] = (float)(2.0 * ((double)yh[i] - (double)y[i]) / acc[1]);
+  if (i < n) dy[i] = (float)(((double)yh[i] - (double)y[i]) * scale);
 }
 
 __global__ void k_adam(long long n, float* __restrict__ p, const float* __restrict__ gr, float* __restrict__ m1,
@@ -871,6 +876,287 @@ __global__ void k_adam(long long n, float* __restrict__ p, const float* __restri
   m1[i] = a;
   m2[i] = b;
   p[i] -= lr * (a / c1) / (sqrtf(b / c2) + eps);
+}
+
+// ---------------------------------------------------------------------------
+// Backward pointwise pass for C = 32 channels.  One block walks over image
+// rows (y, sample) of one 128-pixel column range and does, per tile,
+//   dv = W^T dz + X F^T          (the pointwise and the spectral adjoint)
+//   dz' = dv gelu'(z)            (hidden layers), written out
+//   dW' += dz' v^T, db' += dz'   (gradients of the layer below)
+// so that dz, z and v are read once and dz' is written once: separate kernels
+// for the two products, the GELU, the weight gradient and the bias gradient
+// moved 13 activations of 4 S C H W bytes per layer where this moves four.
+// Products on the bfloat16 tensor cores (m16n8k16, float32 accumulation), the
+// operands and the order of the products as in k_gemm: W^T dz and X F^T in
+// accumulators of their own, K ascending in steps of 16, then added, so dz'
+// is bit for bit what the separate products gave.  The weight gradient stays
+// in registers over all of a block's tiles; the blocks' partial sums are
+// added in a fixed order by k_bwd_reduce.
+// Memory-bound: four activations of 134 MB per layer at 4 x 512 x 512.
+// Measured there (loss and gradient, without the copy to the host): 13.0 ms
+// with the separate kernels, 3.3 ms with this pass; the largest parts had
+// been the bias sums (one block per channel) and the split-K gradient products
+// (64 x 64 tiles of which a quarter was used).
+// Width 32 and at most 64 spectral columns, the sizes the tiles are made for;
+// other networks keep the separate products.
+// ---------------------------------------------------------------------------
+enum { BWD_HIDDEN = 0, BWD_TOP = 1, BWD_LIFT = 2, BWD_OUTER = 3 };
+constexpr int kBwC = 32, kBwPx = 128, kBwP = kBwPx + 8, kBwWP = kBwC + 8, kBwKX = 64, kBwXP = kBwKX + 8;
+constexpr size_t kBwSmem = sizeof(__nv_bfloat16) * (3 * kBwC * kBwP + kBwC * kBwWP + kBwC * kBwXP + kBwKX * kBwP);
+constexpr int kBwPart = kBwC * kBwC + kBwC;   // a block's partial sums: dW', db'
+
+struct BwdArgs {
+  int H, W, R;               // rows R = samples * H
+  int K2;                    // 2 Mx (<= kBwKX)
+  const float* A;            // W [32][32] (hidden, lift) or Q [3][32] (top)
+  const float* X;            // spectral rows [sample][32][H][K2]
+  const float* F;            // [W][K2]
+  const float* din;          // dz [sample][32][H][W], or dy [sample][3][H][W] (top, outer)
+  const float* z;            // (hidden)
+  const float* v;            // input of the layer below, 32 channels (lift: u, 3 channels)
+  float* dout;               // (hidden, top)
+  float* part;               // [block][kBwPart]
+};
+
+__device__ __forceinline__ void ldsm4(unsigned (&r)[4], const __nv_bfloat16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((unsigned)__cvta_generic_to_shared(p))
+               : "memory");
+}
+__device__ __forceinline__ void ldsm4t(unsigned (&r)[4], const __nv_bfloat16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((unsigned)__cvta_generic_to_shared(p))
+               : "memory");
+}
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+
+// rows [0, rows) of an activation tile (128 pixels from px0 of row `row` of
+// each channel plane) as bfloat16 into t[channel][pixel]; pixels >= nx and
+// the channels up to 32 are zero
+__device__ __forceinline__ void bwd_tile(__nv_bfloat16* t, const float* __restrict__ src, long long plane, int rows,
+                                         int nx, bool vec) {
+  if (vec) {
+    constexpr int Q = kBwPx / 4;
+#pragma unroll 8
+    for (int e = threadIdx.x; e < kBwC * Q; e += 128) {
+      const int c = e / Q, px = 4 * (e % Q);
+      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (c < rows && px < nx) v = *reinterpret_cast<const float4*>(src + c * plane + px);
+      *reinterpret_cast<uint2*>(&t[c * kBwP + px]) = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
+    }
+  } else {
+#pragma unroll 4
+    for (int e = threadIdx.x; e < kBwC * kBwPx; e += 128) {
+      const int c = e / kBwPx, px = e % kBwPx;
+      t[c * kBwP + px] = __float2bfloat16_rn(c < rows && px < nx ? src[c * plane + px] : 0.f);
+    }
+  }
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(128, 4) k_bwd_pw(BwdArgs a) {
+  constexpr bool SPEC = MODE == BWD_HIDDEN || MODE == BWD_LIFT;
+  constexpr int KI = SPEC ? kBwC : 3;                  // channels of din
+  constexpr int KV = MODE == BWD_LIFT ? 3 : kBwC;      // channels of v
+  constexpr int MT = MODE == BWD_OUTER ? 1 : 2;        // 16-row tiles of dz'
+  extern __shared__ __align__(16) __nv_bfloat16 bsm[];
+  __nv_bfloat16* Ds = bsm;                             // din [32][px]
+  __nv_bfloat16* Vs = Ds + kBwC * kBwP;                // v [32][px]
+  __nv_bfloat16* Zs = Vs + kBwC * kBwP;                // dz' [32][px]
+  __nv_bfloat16* As = Zs + kBwC * kBwP;                // W^T (Q^T) [32][32]
+  __nv_bfloat16* Xs = As + kBwC * kBwWP;               // X row [32][K2]
+  __nv_bfloat16* Fs = Xs + kBwC * kBwXP;               // F^T [K2][px]
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int x0 = blockIdx.x * kBwPx, nx = min(kBwPx, a.W - x0), wn = warp * 32;
+  const long long N = (long long)a.H * a.W;
+  const bool vec = (a.W & 3) == 0;
+  const int K2s = (a.K2 + 15) / 16;                    // 16-wide steps of the spectral product
+  if (MODE != BWD_OUTER)
+    for (int e = tid; e < kBwC * kBwC; e += 128) {
+      const int k = e / kBwC, m = e % kBwC;            // A(m, k) = W[k][m]
+      As[m * kBwWP + k] = __float2bfloat16_rn(k < KI ? a.A[k * kBwC + m] : 0.f);
+    }
+  if (SPEC) {
+    for (int e = tid; e < 16 * K2s * kBwPx; e += 128) {
+      const int px = e / (16 * K2s), k = e % (16 * K2s);
+      Fs[k * kBwP + px] = __float2bfloat16_rn(px < nx && k < a.K2 ? a.F[(long long)(x0 + px) * a.K2 + k] : 0.f);
+    }
+    for (int e = tid; e < kBwC * kBwXP; e += 128) Xs[e] = __float2bfloat16_rn(0.f);
+  }
+  float dw[MT][4][4], db[MT][2];
+#pragma unroll
+  for (int i = 0; i < MT; ++i) {
+    db[i][0] = db[i][1] = 0.f;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) dw[i][j][r] = 0.f;
+  }
+  // ldmatrix row addresses of this lane: A (16 x 16) at row lane % 16, column
+  // 8 (lane / 16); transposed B (16 k x 16 n) the same; B from [n][k] storage
+  // (16 n x 16 k): row lane % 8 + 8 (lane / 16), column 8 ((lane / 8) & 1)
+  const int ar = lane & 15, ac = 8 * (lane >> 4), br = (lane & 7) + 8 * (lane >> 4), bc = 8 * ((lane >> 3) & 1);
+  for (int row = blockIdx.y; row < a.R; row += gridDim.y) {
+    const int s = row / a.H, y = row % a.H;
+    const long long o = (long long)y * a.W + x0;
+    __syncthreads();   // (the previous tile has been used)
+    bwd_tile(MODE == BWD_OUTER ? Zs : Ds, a.din + (long long)s * KI * N + o, N, KI, nx, vec);
+    bwd_tile(Vs, a.v + (long long)s * KV * N + o, N, KV, nx, vec);
+    if (SPEC)
+      for (int e = tid; e < kBwC * a.K2; e += 128) {
+        const int c = e / a.K2, k = e % a.K2;
+        Xs[c * kBwXP + k] = __float2bfloat16_rn(a.X[(((long long)s * kBwC + c) * a.H + y) * a.K2 + k]);
+      }
+    __syncthreads();
+    if constexpr (MODE == BWD_OUTER) {
+      // (row sums of dy in float32: channel g, the lane's pixels of the warp's range)
+      if (g < KI) {
+        const float* d = a.din + ((long long)s * KI + g) * N + o;
+#pragma unroll
+        for (int p = 0; p < 8; ++p) {
+          const int px = wn + 4 * p + t;
+          if (px < nx) db[0][0] += d[px];
+        }
+      }
+    } else {
+      float p1[2][4][4], p2[2][4][4];
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int r = 0; r < 4; ++r) p1[i][j][r] = p2[i][j][r] = 0.f;
+#pragma unroll
+      for (int ks = 0; ks < (SPEC ? 2 : 1); ++ks) {
+        unsigned af[2][4], bf[2][4];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) ldsm4(af[i], &As[(16 * i + ar) * kBwWP + 16 * ks + ac]);
+#pragma unroll
+        for (int jj = 0; jj < 2; ++jj) ldsm4t(bf[jj], &Ds[(16 * ks + ar) * kBwP + wn + 16 * jj + ac]);
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) mma_bf16(p1[i][j], af[i], bf[j >> 1][2 * (j & 1)], bf[j >> 1][2 * (j & 1) + 1]);
+      }
+      if (SPEC) {
+        for (int ks = 0; ks < K2s; ++ks) {
+          unsigned af[2][4], bf[2][4];
+#pragma unroll
+          for (int i = 0; i < 2; ++i) ldsm4(af[i], &Xs[(16 * i + ar) * kBwXP + 16 * ks + ac]);
+#pragma unroll
+          for (int jj = 0; jj < 2; ++jj) ldsm4t(bf[jj], &Fs[(16 * ks + ar) * kBwP + wn + 16 * jj + ac]);
+#pragma unroll
+          for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              mma_bf16(p2[i][j], af[i], bf[j >> 1][2 * (j & 1)], bf[j >> 1][2 * (j & 1) + 1]);
+        }
+      }
+      // dz' at (channel 16 i + g + 8 q, pixels px, px + 1)
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const int c = 16 * i + g + 8 * q;
+          const long long cb = ((long long)s * kBwC + c) * N + o;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int px = wn + 8 * j + 2 * t;
+            float d0 = p1[i][j][2 * q], d1 = p1[i][j][2 * q + 1];
+            if (SPEC) {
+              d0 = p2[i][j][2 * q] + d0;
+              d1 = p2[i][j][2 * q + 1] + d1;
+            }
+            if (vec) {
+              if (px < nx) {   // (nx is a multiple of 4)
+                if (MODE == BWD_HIDDEN) {
+                  const float2 zz = *reinterpret_cast<const float2*>(a.z + cb + px);
+                  d0 *= gelu_df(zz.x);
+                  d1 *= gelu_df(zz.y);
+                }
+                if (MODE != BWD_LIFT) *reinterpret_cast<float2*>(a.dout + cb + px) = make_float2(d0, d1);
+              }
+            } else {
+              if (px < nx) {
+                if (MODE == BWD_HIDDEN) d0 *= gelu_df(a.z[cb + px]);
+                if (MODE != BWD_LIFT) a.dout[cb + px] = d0;
+              }
+              if (px + 1 < nx) {
+                if (MODE == BWD_HIDDEN) d1 *= gelu_df(a.z[cb + px + 1]);
+                if (MODE != BWD_LIFT) a.dout[cb + px + 1] = d1;
+              }
+            }
+            // (pixels past the image are zero: zero operands)
+            db[i][q] += d0 + d1;
+            *reinterpret_cast<unsigned*>(&Zs[c * kBwP + px]) = pack_bf16(d0, d1);
+          }
+        }
+      __syncwarp();
+    }
+    // dW' += dz' v^T over the warp's 32 pixels
+#pragma unroll
+    for (int ks = 0; ks < 2; ++ks) {
+      unsigned af[MT][4], bf[2][4];
+#pragma unroll
+      for (int i = 0; i < MT; ++i) ldsm4(af[i], &Zs[(16 * i + ar) * kBwP + wn + 16 * ks + ac]);
+#pragma unroll
+      for (int jj = 0; jj < (KV > 16 ? 2 : 1); ++jj) ldsm4(bf[jj], &Vs[(16 * jj + br) * kBwP + wn + 16 * ks + bc]);
+#pragma unroll
+      for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int j = 0; j < (KV > 16 ? 4 : 1); ++j)
+          mma_bf16(dw[i][j], af[i], bf[j >> 1][2 * (j & 1)], bf[j >> 1][2 * (j & 1) + 1]);
+    }
+  }
+  // the block's partial sums: the four warps in order
+  __syncthreads();
+  float* red = reinterpret_cast<float*>(bsm);          // [warp][kBwPart]
+  for (int e = tid; e < 4 * kBwPart; e += 128) red[e] = 0.f;
+  __syncthreads();
+  float* mine = red + warp * kBwPart;
+#pragma unroll
+  for (int i = 0; i < MT; ++i) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        mine[(16 * i + g + (r >= 2 ? 8 : 0)) * kBwC + 8 * j + 2 * t + (r & 1)] = dw[i][j][r];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      float v = db[i][q];
+      v += __shfl_xor_sync(0xffffffffu, v, 1);
+      v += __shfl_xor_sync(0xffffffffu, v, 2);
+      if (t == 0) mine[kBwC * kBwC + 16 * i + g + 8 * q] = v;
+    }
+  }
+  __syncthreads();
+  float* out = a.part + ((long long)blockIdx.y * gridDim.x + blockIdx.x) * kBwPart;
+  for (int e = tid; e < kBwPart; e += 128)
+    out[e] = ((red[e] + red[kBwPart + e]) + red[2 * kBwPart + e]) + red[3 * kBwPart + e];
+}
+
+// dW[m][n] += sum over blocks of part[block][m 32 + n], db[m] likewise (m < M,
+// n < N); one warp per value, lanes over the blocks, a fixed order
+__global__ void k_bwd_reduce(int blocks, int M, int N, const float* __restrict__ part, float* __restrict__ dW,
+                             float* __restrict__ db) {
+  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (w >= M * N + M) return;
+  const int e = w < M * N ? (w / N) * kBwC + w % N : kBwC * kBwC + (w - M * N);
+  float v = 0.f;
+  for (int b = lane; b < blocks; b += 32) v += part[(long long)b * kBwPart + e];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) {
+    if (w < M * N) dW[w] += v;
+    else db[w - M * N] += v;
+  }
 }
 
 // u = (Msat(cell) / ms_ref) m  and  B = mu0 ms_ref y
@@ -937,6 +1223,8 @@ struct mm_fno {
   float2 *O = nullptr, *dO = nullptr, *dV = nullptr;
   float2* Yp = nullptr;                     // row-range partials of the y product
   double* acc = nullptr;
+  bool bwd_pw = false;                      // the fused backward pass serves (C, 2 Mx)
+  float* part = nullptr;                    // its blocks' partial sums
 };
 
 namespace {
@@ -1009,6 +1297,52 @@ void fwd(mm_fno* f, int S) {
     gemm(s, false, false, S, gargs(3, (int)N, C, P_(f, q), C, 0, f->v[L], N, CN, f->yh, N, 3 * N, 1.f, 0.f, P_(f, qq)));
 }
 
+// grid of the fused backward pass: about four blocks per multiprocessor (its
+// residency), each walking over rows of its 128-pixel range
+dim3 bwd_grid(const mm_fno* f, int S) {
+  const int gx = (f->W + kBwPx - 1) / kBwPx;
+  const int gy = std::max(1, std::min(S * f->H, 4 * f->sms / gx));
+  return dim3(gx, gy);
+}
+size_t bwd_part_floats(const mm_fno* f) {
+  const int gx = (f->W + kBwPx - 1) / kBwPx;
+  return (size_t)std::max(gx, 4 * f->sms) * kBwPart;
+}
+template <int MODE>
+void bwd_pw(mm_fno* f, int S, const float* A, const float* X, const float* din, const float* z, const float* v,
+            float* dout, int M, int N, float* dW, float* db) {
+  BwdArgs a{f->H, f->W, S * f->H, 2 * f->Mx, A, X, f->Fblk, din, z, v, dout, f->part};
+  const dim3 grid = bwd_grid(f, S);
+  k_bwd_pw<MODE><<<grid, 128, kBwSmem, f->stream>>>(a);
+  k_bwd_reduce<<<(M * N + M + 7) / 8, 256, 0, f->stream>>>((int)(grid.x * grid.y), M, N, f->part, dW, db);
+}
+template <int MODE>
+bool bwd_attr() {
+  return cudaFuncSetAttribute(k_bwd_pw<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBwSmem) == cudaSuccess;
+}
+// whether the fused backward pass serves this width and mode count (raises
+// its shared-memory limit; called at creation)
+bool bwd_prepare(int C, int K2) {
+  if (C != kBwC || K2 > kBwKX) return false;
+  const bool ok = bwd_attr<BWD_HIDDEN>() && bwd_attr<BWD_TOP>() && bwd_attr<BWD_LIFT>() && bwd_attr<BWD_OUTER>();
+  if (!ok) (void)cudaGetLastError();
+  return ok;
+}
+
+// the spectral adjoint of layer l: dR and the rows X of dV Fy^T from dz
+void bwd_spectral(mm_fno* f, int S, int l, const float* dzl, const YTile& yt, int xp) {
+  cudaStream_t s = f->stream;
+  const int C = f->C, H = f->H, W = f->W, Mx = f->Mx, J = f->J;
+  gemm(s, false, true, S, sliced(gargs(C * H, 2 * Mx, W, dzl, W, (long long)C * f->N, f->Gblk, W, 0, f->Z, 2 * Mx,
+                                       (long long)C * H * 2 * Mx), xp, f->xslice));
+  ysum(s, yt, S, C, H, J, Mx, f->Z, true, xp, f->xslice, f->Gy, true, f->dO, f->Yp);
+  k_dR<<<nb((long long)C * C * J * Mx), 256, 0, s>>>(S, C, J * Mx, f->dO, f->V[l],
+                                                    reinterpret_cast<float2*>(G_(f, sR(l))));
+  k_mix<<<mix_blocks((long long)S * C * J * Mx), 256, 0, s>>>(S, C, J * Mx, reinterpret_cast<const float2*>(P_(f, sR(l))),
+                                                    f->dO, f->dV, true);
+  yexpand(s, yt, S, C, H, J, Mx, f->dV, f->Fy, true, f->X);
+}
+
 // gradients of the batch loss into f->grd (zeroed here); loss pieces in acc
 void bwd(mm_fno* f, int S, const float* y) {
   cudaStream_t s = f->stream;
@@ -1021,6 +1355,22 @@ void bwd(mm_fno* f, int S, const float* y) {
   cudaMemsetAsync(f->acc, 0, 2 * sizeof(double), s);
   k_loss<<<1024, 256, 0, s>>>(S * 3 * N, f->yh, y, f->acc);
   k_dloss<<<nb(S * 3 * N), 256, 0, s>>>(S * 3 * N, f->yh, y, f->acc, f->dy);
+  if (f->bwd_pw) {
+    // one pass over the activations per layer (k_bwd_pw)
+    bwd_pw<BWD_OUTER>(f, S, nullptr, nullptr, f->dy, nullptr, f->v[L], nullptr, 3, C, G_(f, sW(L)), G_(f, sb(L)));
+    bwd_pw<BWD_TOP>(f, S, P_(f, sW(L)), nullptr, f->dy, nullptr, f->v[L - 1], f->dv, C, C, G_(f, sW(L - 1)),
+                    G_(f, sb(L - 1)));
+    for (int l = L - 1; l >= 0; --l) {
+      bwd_spectral(f, S, l, f->dv, yt, xp);
+      if (l > 0)
+        bwd_pw<BWD_HIDDEN>(f, S, P_(f, sW(l)), f->X, f->dv, f->z[l - 1], f->v[l - 1], f->dv2, C, C, G_(f, sW(l - 1)),
+                           G_(f, sb(l - 1)));
+      else
+        bwd_pw<BWD_LIFT>(f, S, P_(f, sW(0)), f->X, f->dv, nullptr, f->u, nullptr, C, 3, G_(f, 0), G_(f, 1));
+      std::swap(f->dv, f->dv2);
+    }
+    return;
+  }
   // project
   for (int b = 0; b < S; ++b)
     gemm(s, false, true, 1, gargs(3, C, (int)N, f->dy + b * 3 * N, N, 0, f->v[L] + b * CN, N, 0, G_(f, sW(L)), C, 0,
@@ -1036,15 +1386,7 @@ void bwd(mm_fno* f, int S, const float* y) {
     k_rowsum<<<C, 256, 0, s>>>(S, C, N, dzl, G_(f, sb(l)));
     // dv2 = W^T dz
     gemm(s, true, false, S, gargs(C, (int)N, C, P_(f, sW(l)), C, 0, dzl, N, CN, f->dv2, N, CN));
-    // spectral adjoint: dZ_blk = dz [C H x W] . Gblk^T
-    gemm(s, false, true, S, sliced(gargs(C * H, 2 * Mx, W, dzl, W, CN, f->Gblk, W, 0, f->Z, 2 * Mx,
-                                         (long long)C * H * 2 * Mx), xp, f->xslice));
-    ysum(s, yt, S, C, H, J, Mx, f->Z, true, xp, f->xslice, f->Gy, true, f->dO, f->Yp);
-    k_dR<<<nb((long long)C * C * J * Mx), 256, 0, s>>>(S, C, J * Mx, f->dO, f->V[l],
-                                                      reinterpret_cast<float2*>(G_(f, sR(l))));
-    k_mix<<<mix_blocks((long long)S * C * J * Mx), 256, 0, s>>>(S, C, J * Mx, reinterpret_cast<const float2*>(P_(f, sR(l))),
-                                                      f->dO, f->dV, true);
-    yexpand(s, yt, S, C, H, J, Mx, f->dV, f->Fy, true, f->X);
+    bwd_spectral(f, S, l, dzl, yt, xp);
     // dv2 += dX_blk [C H x 2Mx] . Fblk^T [2Mx x W]
     gemm(s, false, true, S, gargs(C * H, W, 2 * Mx, f->X, 2 * Mx, (long long)C * H * 2 * Mx, f->Fblk, 2 * Mx, 0, f->dv2,
                                   W, CN, 1.f, 1.f));
@@ -1074,6 +1416,7 @@ int mm_fno_create(mm_fno** out, int H, int W, const mm_fno_cfg* cfg, int device,
   f->device = device;
   f->sms = sms;
   f->layer_pw = layer_pw_prepare(C, 2 * Mx);
+  f->bwd_pw = bwd_prepare(C, 2 * Mx);
   f->C = C; f->L = L; f->Mx = Mx; f->My = My; f->H = H; f->W = W; f->J = 2 * My; f->Smax = Smax;
   f->N = (long long)H * W;
   auto cleanup = [&](int code) { mm_fno_destroy(f); return code; };
@@ -1125,6 +1468,7 @@ int mm_fno_create(mm_fno** out, int H, int W, const mm_fno_cfg* cfg, int device,
   alloc((void**)&f->dV, (size_t)Smax * C * f->J * Mx * sizeof(float2));
   alloc((void**)&f->Yp, (size_t)kYSplit * Smax * C * f->J * Mx * sizeof(float2));
   alloc((void**)&f->acc, 4 * sizeof(double));
+  if (f->bwd_pw) alloc((void**)&f->part, bwd_part_floats(f) * sizeof(float));
   if (e != cudaSuccess) return cleanup(ffail(e == cudaErrorMemoryAllocation ? MM_ERR_OOM : MM_ERR_CUDA, cudaGetErrorString(e)));
   // partial DFT matrices (float64 on the host, rounded once)
   const double pi = 3.14159265358979323846;
@@ -1184,7 +1528,7 @@ int mm_fno_destroy(mm_fno* f) {
   cudaSetDevice(f->device);
   if (f->stream) cudaStreamSynchronize(f->stream);
   void* ptrs[] = {f->prm, f->grd, f->m1, f->m2, f->Fblk, f->Gblk, f->Fy, f->Gy, f->u, f->yh, f->dy,
-                  f->X, f->Z, f->dv, f->dv2, f->O, f->dO, f->dV, f->Yp, f->acc};
+                  f->X, f->Z, f->dv, f->dv2, f->O, f->dO, f->dV, f->Yp, f->acc, f->part};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   for (float* p : f->v) if (p) cudaFree(p);
