@@ -15,7 +15,8 @@ OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libmm.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 UNITS = ["demag_tensor.cu", "fft_conv.cu", "fft_fused.cu", "llg.cu", "mm_api.cu", "demag_noalloc.cu", "batch.cu", "fno.cu", "rowstage.cu", "peak.cu", "fft_yz3.cu",
-         "film.cu", "film_l16.cu", "film_l32.cu", "film_l64.cu", "film_l128.cu", "film_l256.cu", "film_l512.cu"]
+         "film.cu", "film_l16.cu", "film_l32.cu", "film_l64.cu", "film_l128.cu", "film_l256.cu", "film_l512.cu",
+         "film3_l16.cu", "film3_l32.cu", "film3_l64.cu", "film3_l128.cu", "film3_l256.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", f"-I{INCLUDE}"]
 

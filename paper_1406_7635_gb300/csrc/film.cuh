@@ -185,28 +185,42 @@ __device__ __forceinline__ float2 swapc(float2 a) { return make_float2(a.y, a.x)
 // Work split for rows of LX complex values and PH points per y class: ROWS
 // film rows per block, CPB columns per block so that at most kFilmBlocks
 // blocks hold the LX + 1 columns, QR of them transformed at a time.
+// PZ: 1 for films; the padded z length of thin 3-D grids (two to four
+// layers), whose blocks own rows of one layer and whole (y, z) planes of kx.
 constexpr int kFilmBlocks = 148;
-template <int LX, int PH, int ROWS>
+template <int LX, int PH, int ROWS, int PZ>
 struct FilmCfg {
   using FX = FilmFft<LX>;
   using FY = FilmFft<PH>;
   static constexpr int CPB = (LX + 1 + kFilmBlocks - 1) / kFilmBlocks;
-  static constexpr int NTC = ROWS * LX, NTY = 6 * CPB * FY::LANES;   // one cell, one column lane per thread
+  static constexpr int NZ = PZ > 1 ? PZ / 2 : 1;   // most layers
+  static constexpr int NTC = ROWS * LX, NTY = 6 * NZ * CPB * FY::LANES;   // one cell, one column lane per thread
   static constexpr int NT0 = ((NTC > NTY ? NTC : NTY) + 31) / 32 * 32;
   static constexpr int NT = NT0 < 64 ? 64 : (NT0 > 512 ? 512 : NT0);
   static constexpr int QR0 = NT / (6 * FY::LANES);
-  static constexpr int QR = QR0 < 1 ? 1 : (QR0 > CPB ? CPB : QR0);
+  static constexpr int QR = PZ > 1 || QR0 < 1 ? 1 : (QR0 > CPB ? CPB : QR0);
   // cells per thread: up to four, enough for periodic rows (2 LX cells) except
   // three or more of the longest
   static constexpr int CELLS0 = (2 * NTC + NT - 1) / NT;
   static constexpr int CELLS = CELLS0 > 4 ? 4 : CELLS0;
-  static constexpr int LANX = (3 * ROWS * FX::LANES + 31) / 32 * 32, LANY = (6 * QR * FY::LANES + 31) / 32 * 32;
-  static_assert(LANX <= NT && LANY <= NT, "every pencil has its lanes");
+  static constexpr int LR = PZ > 1 ? 3 * ROWS + 2 : ROWS + 2;   // stencil rows
+  static constexpr int ND = PZ > 1 ? 6 : 4;                     // stencil directions
+  static constexpr int LANX = (3 * ROWS * FX::LANES + 31) / 32 * 32;
+  // column pencils transformed at a time, in rounds of NT lanes
+  static constexpr int PPW = 32 / FY::LANES;                    // per warp
+  static constexpr int NPEN = (6 * NZ * QR + PPW - 1) / PPW * PPW;
+  static_assert(LANX <= NT, "every row pencil has its lanes");
   // pencil areas (whole warps have one, so that idle lanes have a place to work)
-  static constexpr int NX = LANX / FX::LANES * FX::AREA, NY = LANY / FY::LANES * FY::AREA;
+  static constexpr int NX = LANX / FX::LANES * FX::AREA, NY = NPEN * FY::AREA;
   static constexpr int FFT = NX > NY ? NX : NY;
   static constexpr int TAB = FX::TAB + (LX + 1) + FY::TAB + PH;
-  static constexpr int OCT = CPB * 4 * (PH + 1);
+  // octant values per column: xx, yy, zz, xy (one layer: Kxz and Kyz are odd
+  // in z and vanish at kz = 0), or all six at PZ / 2 + 1 frequencies
+  static constexpr int OCOL = (PZ > 1 ? 6 * (PZ / 2 + 1) : 4) * (PH + 1);
+  static constexpr int OCT = CPB * OCOL;
+  // stage rows: films keep two buffers (the next input is written while the
+  // stencil reads this one); 3-D grids one, refilled from global memory
+  static constexpr int STG = PZ > 1 ? 1 : 2;
 };
 
 __device__ __forceinline__ void red_release(unsigned int* p) {
@@ -245,31 +259,36 @@ __device__ __forceinline__ double film_stage_time(double t, double h, int method
   return s < 3 || s == 6 ? t + kC23[s == 6 ? 3 : s] * h : t;
 }
 
-template <int LX, int PH, int ROWS>
-__global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS>::NT, 1) k_film(const __grid_constant__ FilmArgs a) {
-  using F = FilmCfg<LX, PH, ROWS>;
+template <int LX, int PH, int ROWS, int PZ>
+__global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS, PZ>::NT, 1) k_film(const __grid_constant__ FilmArgs a) {
+  using F = FilmCfg<LX, PH, ROWS, PZ>;
   using FX = typename F::FX;
   using FY = typename F::FY;
-  constexpr int NT = F::NT, CPB = F::CPB, QR = F::QR, LR = ROWS + 2, CELLS = F::CELLS;
+  constexpr int NT = F::NT, CPB = F::CPB, QR = F::QR, LR = F::LR, CELLS = F::CELLS;
+  constexpr int ND = F::ND;
+  constexpr bool D3 = PZ > 1;
   const Geom& g = a.g;
   const int nx = g.nx, ny = g.ny, n = (int)g.n, tid = threadIdx.x, lane = tid & 31;
   constexpr int hx = LX + 1;
-  const int y0 = blockIdx.x * ROWS, kx0 = blockIdx.x * CPB;
-  const int nrow = max(0, min(ROWS, ny - y0)), ncol = max(0, min(CPB, hx - kx0));
+  // rows y0 .. of layer z
+  const int nz = D3 ? g.nz : 1, nch = (ny + ROWS - 1) / ROWS;
+  const int z = D3 ? blockIdx.x / nch : 0, y0 = (D3 ? blockIdx.x % nch : blockIdx.x) * ROWS;
+  const int kx0 = blockIdx.x * CPB;
+  const int nrow = z < nz ? max(0, min(ROWS, ny - y0)) : 0, ncol = max(0, min(CPB, hx - kx0));
   const int ncell = nrow * nx, D = LR * nx;
 
   extern __shared__ float4 film_dyn[];
   // (the stage rows first: with nx a multiple of 4 they take 16-byte copies)
-  float* sst = reinterpret_cast<float*>(film_dyn);            // stage input, two buffers [3][LR][nx]
-  float2* fb = reinterpret_cast<float2*>(sst + 2 * 3 * D);    // pencil areas (6 D floats before: 8-byte aligned)
+  float* sst = reinterpret_cast<float*>(film_dyn);            // stage input, STG buffers [3][LR][nx]
+  float2* fb = reinterpret_cast<float2*>(sst + (F::STG * 3 * D + 1) / 2 * 2);   // pencil areas (8-byte aligned)
   float2* tx = fb + F::FFT;                                   // x twiddles
   float2* ty = tx + FX::TAB;                                  // y twiddles
   float2* twc = ty + FY::TAB;                                 // W_2PH^y (class 1)
   float2* tw2 = twc + PH;                                     // W_2LX^k, k <= LX
   RegionLUT* lut = reinterpret_cast<RegionLUT*>(tw2 + LX + 1);
-  float* ce = reinterpret_cast<float*>(lut + 1);              // exchange couplings [4][ROWS nx]
-  int* sco = reinterpret_cast<int*>(ce + 4 * ROWS * nx);      // codes [LR][nx]
-  float* soct = reinterpret_cast<float*>(sco + LR * nx);      // octant [CPB][xx, yy, zz, xy][PH + 1]
+  float* ce = reinterpret_cast<float*>(lut + 1);              // exchange couplings [ND][ROWS nx]
+  int* sco = reinterpret_cast<int*>(ce + ND * ROWS * nx);      // codes [LR][nx]
+  float* soct = reinterpret_cast<float*>(sco + LR * nx);      // octant [CPB][component, kz][PH + 1]
   __shared__ DevState S;
   __shared__ StageCoef sc;
   __shared__ float sinv[7];
@@ -283,16 +302,27 @@ __global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS>::NT, 1) k_film(const __g
   for (int i = tid; i <= LX; i += NT) tw2[i] = __ldg(&a.tw[(i * (kTwN / (2 * LX))) & (kTwN - 1)]);
   for (int i = tid; i < (int)(sizeof(RegionLUT) / 4); i += NT)
     reinterpret_cast<float*>(lut)[i] = __ldg(reinterpret_cast<const float*>(a.lut) + i);
+  // stencil row lr: own layer from y0 - 1 (ROWS + 2 rows), then rows y0 .. of
+  // the layer below, then of the layer above; -1 outside the grid
+  auto stencil_row = [&](int lr) -> int {
+    int yy = y0 - 1 + lr, zz = z;
+    if (D3 && lr >= ROWS + 2) {
+      const int q = lr - (ROWS + 2);
+      yy = y0 + q % ROWS;
+      zz = q < ROWS ? z - 1 : z + 1;
+    }
+    return yy >= 0 && yy < ny && zz >= 0 && zz < nz ? zz * ny + yy : -1;
+  };
   for (int e = tid; e < LR * nx; e += NT) {
-    const int y = y0 - 1 + e / nx;
-    sco[e] = (y >= 0 && y < ny) ? a.code[y * nx + e % nx] : kVacuum;
+    const int row = stencil_row(e / nx);
+    sco[e] = row >= 0 ? a.code[row * nx + e % nx] : kVacuum;
   }
-  // one layer: Kxz and Kyz are odd in z and vanish at kz = 0
-  const int per = g.hky;   // (hkz = 1)
+  const int per = g.hky * g.hkz;
   if (a.oct_sm)
-    for (int e = tid; e < ncol * 4 * (PH + 1); e += NT) {
-      const int i = e % (PH + 1), t = (e / (PH + 1)) & 3, q = e / (4 * (PH + 1));
-      soct[e] = __ldg(&a.kt[((kx0 + q) * 6 + t) * per + i]);
+    for (int e = tid; e < ncol * F::OCOL; e += NT) {
+      const int q = e / F::OCOL, i = e % F::OCOL;
+      // (the components of a column are contiguous: films take the first four)
+      soct[e] = __ldg(&a.kt[(kx0 + q) * 6 * per + i]);
     }
   for (int i = tid; i < (int)(sizeof(DevState) / 4); i += NT)
     reinterpret_cast<unsigned*>(&S)[i] = __ldcg(reinterpret_cast<const unsigned*>(a.st) + i);
@@ -309,28 +339,33 @@ __global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS>::NT, 1) k_film(const __g
       }
   };
   // stencil positions of own cell (r, x): a missing neighbour is the cell
-  // itself; the two z neighbours are too (one layer)
-  auto neighbours = [&](int r, int x, int (&nb)[4]) {
+  // itself (one layer: both z neighbours, not visited)
+  auto neighbours = [&](int r, int x, int (&nb)[ND]) {
     const int y = y0 + r, C = (r + 1) * nx + x;
     nb[0] = x > 0 ? C - 1 : (g.pbcx ? C + nx - 1 : C);
     nb[1] = x < nx - 1 ? C + 1 : (g.pbcx ? C - (nx - 1) : C);
     nb[2] = y > 0 ? C - nx : C;
     nb[3] = y < ny - 1 ? C + nx : C;
+    if constexpr (D3) {
+      nb[4] = z > 0 ? (ROWS + 2 + r) * nx + x : C;
+      nb[5] = z < nz - 1 ? (2 * ROWS + 2 + r) * nx + x : C;
+    }
   };
   // exchange couplings of the own cells, 2 S H(Aex / Msat) / d^2 per direction
   // (with DMI a missing neighbour is a ghost coupled like the cell itself)
   for (int e = tid; e < ncell; e += NT) {
-    int r, x, nb[4];
+    int r, x, nb[ND];
     split(e, r, x);
     neighbours(r, x, nb);
     const int C = (r + 1) * nx + x, ci = sco[C];
 #pragma unroll
-    for (int d = 0; d < 4; ++d) {
+    for (int d = 0; d < ND; ++d) {
       const int cj = sco[nb[d]];
       const bool present = (nb[d] != C || (g.pbcx && d < 2)) && cj != kVacuum;
       float c = 0.0f;
       if (ci != kVacuum && (a.T.dmi ? a.T.exch : 1))
-        c = __ldg(&a.xlut[ci * kXStride + (a.T.dmi && !present ? ci : cj)]) * (d < 2 ? g.idx2 : g.idy2);
+        c = __ldg(&a.xlut[ci * kXStride + (a.T.dmi && !present ? ci : cj)]) *
+            (d < 2 ? g.idx2 : (d < 4 ? g.idy2 : g.idz2));
       ce[d * ROWS * nx + e] = c;
     }
   }
@@ -386,7 +421,7 @@ __global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS>::NT, 1) k_film(const __g
   }
 
   // m and the k's stay in the global buffers; a thread reads only what it wrote
-  const int own = y0 * nx;   // first own cell
+  const int own = (z * ny + y0) * nx;   // first own cell
   auto kbuf = [&](int j) -> float* {
     float* p;
     switch (j) {
@@ -451,15 +486,15 @@ __global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS>::NT, 1) k_film(const __g
     float* __restrict__ mcur = (par ? a.m1 : a.m0) + own;
     int cur = 0;   // stage buffer in use
     if (blockIdx.x == 0 && tid == 0) a.sync->err[(att + 1) % 3] = 0;
-    // a cell's stage input: stage buffer, halo rows for the neighbours, M in
-    // the row pencils
+    // a cell's stage input: stage buffer (3-D: filled from the halo array later),
+    // rows for the neighbours, M in the row pencils
     auto put = [&](float* st_, int e, int r, int x, int ci, const float (&v)[3]) {
       const float ms = ci != kVacuum ? lut->msat[ci] : 0.f;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        st_[c * D + (r + 1) * nx + x] = v[c];
+        if (!D3) st_[c * D + (r + 1) * nx + x] = v[c];
         rowf[rix(c, r, x)] = ms * v[c];
-        if (r == 0 || r == nrow - 1) a.halo[c * n + own + e] = v[c];
+        if (D3 || r == 0 || r == nrow - 1) a.halo[c * n + own + e] = v[c];
       }
     };
     {   // the input of the second stage (k1: of the first, m itself)
@@ -504,16 +539,17 @@ __global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS>::NT, 1) k_film(const __g
           if (r >= nrow) continue;
           const float2* row = fb + (c * ROWS + r) * FX::AREA;
           const float2 zk = row[FX::pos(k)], zl = k ? row[FX::pos(LX - k)] : zk;
-          float2* dst = a.spec1 + c * hx * ny + y0 + r;
+          const int ks = nz * ny;   // stride of kx in spec1
+          float2* dst = a.spec1 + c * hx * ks + z * ny + y0 + r;
           {
             const float2 zc = cconj(zl);
             const float2 E = cscale(cadd(zk, zc), 0.5f), d = csub(zk, zc);
-            dst[k * ny] = cadd(E, cmul(tw2[k], make_float2(0.5f * d.y, -0.5f * d.x)));
+            dst[k * ks] = cadd(E, cmul(tw2[k], make_float2(0.5f * d.y, -0.5f * d.x)));
           }
           if (k != LX / 2) {
             const float2 zc = cconj(zk);
             const float2 E = cscale(cadd(zl, zc), 0.5f), d = csub(zl, zc);
-            dst[(LX - k) * ny] = cadd(E, cmul(tw2[LX - k], make_float2(0.5f * d.y, -0.5f * d.x)));
+            dst[(LX - k) * ks] = cadd(E, cmul(tw2[LX - k], make_float2(0.5f * d.y, -0.5f * d.x)));
           }
         }
       arrive();
@@ -552,85 +588,98 @@ __global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS>::NT, 1) k_film(const __g
       }
       if (!wait()) return timeout();
       // ---- columns: y forward, kernel product, y inverse ----
-      // (the halo rows of the stencil: their owners wrote them before the barrier)
+      // (the stencil rows of other blocks, in 3-D all of them: their owners
+      // wrote them before the barrier)
       if (nrow > 0) {
-        if ((nx & 3) == 0) {
-          const int cpr = nx / 4;
-          for (int e = tid; e < 6 * cpr; e += NT) {
-            const int ch = e % cpr, q = e / cpr, c = q >> 1, hi = q & 1;
-            const int y = hi ? y0 + nrow : y0 - 1;
-            if (y >= 0 && y < ny) {
-              const unsigned d =
-                  (unsigned)__cvta_generic_to_shared(&st_[c * D + (hi ? nrow + 1 : 0) * nx + 4 * ch]);
-              asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d),
-                           "l"(a.halo + c * n + y * nx + 4 * ch)
-                           : "memory");
-            }
-          }
-        } else {
-          for (int e = tid; e < 6 * nx; e += NT) {
-            const int x = e % nx, q = e / nx, c = q >> 1, hi = q & 1;
-            const int y = hi ? y0 + nrow : y0 - 1;
-            if (y >= 0 && y < ny) {
-              const unsigned d = (unsigned)__cvta_generic_to_shared(&st_[c * D + (hi ? nrow + 1 : 0) * nx + x]);
-              asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(a.halo + c * n + y * nx + x)
-                           : "memory");
-            }
-          }
+        constexpr int NH = D3 ? LR : 2;   // rows to fetch per component
+        const bool vec = (nx & 3) == 0;   // (rows on 16-byte boundaries)
+        const int cpr = vec ? nx / 4 : nx;
+        for (int e = tid; e < 3 * NH * cpr; e += NT) {
+          const int ch = e % cpr, q = e / cpr, c = q / NH, lr = D3 ? q % NH : (q % NH ? nrow + 1 : 0);
+          const int row = stencil_row(lr);
+          if (row < 0) continue;
+          const int w = vec ? 4 * ch : ch;
+          const unsigned d = (unsigned)__cvta_generic_to_shared(&st_[c * D + lr * nx + w]);
+          const float* src = a.halo + c * n + row * nx + w;
+          if (vec) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
+          else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
         }
       }
 #pragma unroll 1
       for (int q0 = 0; q0 < ncol; q0 += QR) {
         if (q0 > 0) __syncthreads();   // (the previous columns' areas are read)
         const int nq = min(QR, ncol - q0);
-        if (tid < F::LANY) {
-          const int q = pc / 6, c = (pc >> 1) % 3, cls = pc & 1;
-          const float2* src = a.spec1 + (c * hx + kx0 + q0 + q) * ny;
-          const bool on = q < nq;
-          FY::run(fb + pc * FY::AREA, ty, jy, [&](int y, int) {
+        const int npen = 6 * nz * nq;
+        // pencil ((q 3 + c) nz + layer) 2 + class
+        for (int p = pc; p < (npen + F::PPW - 1) / F::PPW * F::PPW; p += NT / FY::LANES) {
+          const int cls = p & 1, layer = D3 ? (p >> 1) % nz : 0, cq = (p >> 1) / nz, c = cq % 3, q = cq / 3;
+          const float2* src = a.spec1 + ((c * hx + kx0 + q0 + q) * nz + layer) * ny;
+          const bool on = p < npen;
+          FY::run(fb + p * FY::AREA, ty, jy, [&](int y, int) {
             const float2 v = on && y < ny ? __ldcg(src + y) : make_float2(0.f, 0.f);
             return cls ? cmul(v, twc[y]) : v;
           });
         }
         __syncthreads();
-        // ky = 2 k + class; Kxy is odd in ky
+        // the kernel product at ky = 2 k + class: Kxy is odd in ky, Kxz in kz,
+        // Kyz in both; the result's parts are exchanged (the transform that
+        // follows is the inverse)
+#pragma unroll 1
         for (int e = tid; e < nq * 2 * PH; e += NT) {
           const int k = e % PH, s2 = (e / PH) & 1, q = e / (2 * PH), ky = 2 * k + s2;
           const int iy = ky > PH ? 2 * PH - ky : ky;
-          float kxx, kyy, kzz, kxy;
-          if (a.oct_sm) {
-            const float* o = soct + (q0 + q) * 4 * (PH + 1) + iy;
-            kxx = o[0];
-            kyy = o[PH + 1];
-            kzz = o[2 * (PH + 1)];
-            kxy = o[3 * (PH + 1)];
+          const float sy = ky > PH ? -1.f : 1.f;
+          const float* ko = a.oct_sm ? soct + (q0 + q) * F::OCOL + iy : a.kt + (kx0 + q0 + q) * 6 * per + iy;
+          float2* p = fb + (q * 6 * nz + s2) * FY::AREA + FY::pos(k);   // component c, layer l at (c nz + l) 2 AREA
+          if constexpr (!D3) {
+            const float kxx = ko[0], kyy = ko[PH + 1], kzz = ko[2 * (PH + 1)], kxy = sy * ko[3 * (PH + 1)];
+            const float2 X = p[0], Y = p[2 * FY::AREA], Z = p[4 * FY::AREA];
+            p[0] = make_float2(kxx * X.y + kxy * Y.y, kxx * X.x + kxy * Y.x);
+            p[2 * FY::AREA] = make_float2(kxy * X.y + kyy * Y.y, kxy * X.x + kyy * Y.x);
+            p[4 * FY::AREA] = make_float2(kzz * Z.y, kzz * Z.x);
           } else {
-            const float* o = a.kt + (kx0 + q0 + q) * 6 * per + iy;
-            kxx = __ldg(o);
-            kyy = __ldg(o + per);
-            kzz = __ldg(o + 2 * per);
-            kxy = __ldg(o + 3 * per);
+            // the PZ-point z transforms of the column's layers in registers
+            constexpr int HZ = (PZ / 2 + 1) * (PH + 1);   // octant values per component
+            float2 v[3][PZ];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+#pragma unroll
+              for (int l = 0; l < PZ; ++l)
+                v[c][l] = l < F::NZ && l < nz ? p[(c * nz + l) * 2 * FY::AREA] : make_float2(0.f, 0.f);
+              Dft<PZ, -1>::run(v[c]);
+            }
+#pragma unroll
+            for (int kz = 0; kz < PZ; ++kz) {
+              const float* o = ko + (kz > PZ / 2 ? PZ - kz : kz) * (PH + 1);
+              const float sz = kz > PZ / 2 ? -1.f : 1.f;
+              const float kxx = o[0], kyy = o[HZ], kzz = o[2 * HZ], kxy = sy * o[3 * HZ], kxz = sz * o[4 * HZ],
+                          kyz = sy * sz * o[5 * HZ];
+              const float2 X = v[0][kz], Y = v[1][kz], Z = v[2][kz];
+              v[0][kz] = make_float2(kxx * X.x + kxy * Y.x + kxz * Z.x, kxx * X.y + kxy * Y.y + kxz * Z.y);
+              v[1][kz] = make_float2(kxy * X.x + kyy * Y.x + kyz * Z.x, kxy * X.y + kyy * Y.y + kyz * Z.y);
+              v[2][kz] = make_float2(kxz * X.x + kyz * Y.x + kzz * Z.x, kxz * X.y + kyz * Y.y + kzz * Z.y);
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+              Dft<PZ, 1>::run(v[c]);
+#pragma unroll
+              for (int l = 0; l < F::NZ; ++l)
+                if (l < nz) p[(c * nz + l) * 2 * FY::AREA] = swapc(v[c][l]);
+            }
           }
-          if (ky > PH) kxy = -kxy;
-          float2* p = fb + (q * 6 + s2) * FY::AREA + FY::pos(k);
-          const float2 X = p[0], Y = p[2 * FY::AREA], Z = p[4 * FY::AREA];
-          // (exchanged parts: the transform that follows is the inverse)
-          p[0] = make_float2(kxx * X.y + kxy * Y.y, kxx * X.x + kxy * Y.x);
-          p[2 * FY::AREA] = make_float2(kxy * X.y + kyy * Y.y, kxy * X.x + kyy * Y.x);
-          p[4 * FY::AREA] = make_float2(kzz * Z.y, kzz * Z.x);
         }
         __syncthreads();
-        if (tid < F::LANY) {
-          float2* e = fb + pc * FY::AREA;
+        for (int p = pc; p < (npen + F::PPW - 1) / F::PPW * F::PPW; p += NT / FY::LANES) {
+          float2* e = fb + p * FY::AREA;
           FY::run(e, ty, jy, [&](int i, int) { return e[FY::pos(i)]; });
         }
         __syncthreads();
         // x[y] = x_0[y] + conj(W_2PH^y) x_1[y]; consecutive threads on the
         // block's columns (a run of 8 QR bytes in spec2)
-        for (int e = tid; e < nq * 3 * ny; e += NT) {
-          const int q = e % nq, y = (e / nq) % ny, c = e / (nq * ny);
-          const float2* p = fb + 2 * (q * 3 + c) * FY::AREA + FY::pos(y);
-          a.spec2[(c * ny + y) * g.hxs + kx0 + q0 + q] = cadd(swapc(p[0]), cmul(swapc(p[FY::AREA]), cconj(twc[y])));
+        for (int e = tid; e < nq * 3 * nz * ny; e += NT) {
+          const int q = e % nq, y = (e / nq) % ny, cl = e / (nq * ny);   // cl = c nz + layer
+          const float2* p = fb + 2 * (q * 3 * nz + cl) * FY::AREA + FY::pos(y);
+          a.spec2[(cl * ny + y) * g.hxs + kx0 + q0 + q] = cadd(swapc(p[0]), cmul(swapc(p[FY::AREA]), cconj(twc[y])));
         }
       }
       asm volatile("cp.async.wait_all;\n" ::: "memory");
@@ -641,7 +690,7 @@ __global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS>::NT, 1) k_film(const __g
         for (int e = tid; e < 3 * ROWS * (LX / 2 + 1); e += NT) {
           const int k = e % (LX / 2 + 1), pen = e / (LX / 2 + 1), r = pen % ROWS, c = pen / ROWS;
           if (r >= nrow) continue;
-          const float2* row = a.spec2 + (c * ny + y0 + r) * g.hxs;
+          const float2* row = a.spec2 + ((c * nz + z) * ny + y0 + r) * g.hxs;
           const float2 xa = __ldcg(row + k), xb = __ldcg(row + LX - k);
           float2 za, zb;
           {
@@ -667,14 +716,14 @@ __global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS>::NT, 1) k_film(const __g
       // ---- cells: field, torque, next stage input or error and candidate ----
       const float sinft = a.T.zeeman ? sinv[s] : 0.0f;
       float* ks = kbuf(k_role(s, par));
-      float* nst = sst + (cur ^ 1) * 3 * D;
+      float* nst = sst + (D3 ? 0 : (cur ^ 1) * 3 * D);
       const float wn = s < 6 ? sc.ah[nxt][s] : sc.eh[6];
       float* mnew = (par ? a.m0 : a.m1) + own;
 #pragma unroll
       for (int q = 0; q < CELLS; ++q) {
         const int e = tid + q * NT;
         if (e >= ncell) break;
-        int r, x, nb[4];
+        int r, x, nb[ND];
         split(e, r, x);
         neighbours(r, x, nb);
         const int C = (r + 1) * nx + x, ci = sco[C];
@@ -688,7 +737,7 @@ __global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS>::NT, 1) k_film(const __g
           if (!a.T.dmi) {
             if (a.T.exch) {
 #pragma unroll
-              for (int d = 0; d < 4; ++d) {
+              for (int d = 0; d < ND; ++d) {
                 const float c = ce[d * ROWS * nx + e];
                 ex.x += c * (st_[nb[d]] - mi.x);
                 ex.y += c * (st_[D + nb[d]] - mi.y);
@@ -699,7 +748,7 @@ __global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS>::NT, 1) k_film(const __g
             const float cbc = lut->dbc[ci];
             float3 v[4];
 #pragma unroll
-            for (int d = 0; d < 4; ++d) {
+            for (int d = 0; d < ND; ++d) {
               const int j = nb[d];
               const bool present = (j != C || (g.pbcx && d < 2)) && sco[j] != kVacuum;
               const float3 mj = present ? f3(st_[j], st_[D + j], st_[2 * D + j]) : dmi_ghost(mi, d, cbc, g.cdx, g.cdy);
@@ -707,7 +756,7 @@ __global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS>::NT, 1) k_film(const __g
               ex.x += c * (mj.x - mi.x);
               ex.y += c * (mj.y - mi.y);
               ex.z += c * (mj.z - mi.z);
-              v[d] = mj;
+              if (d < 4) v[d] = mj;
             }
             P.dmi = dmi_field(lut->dmi[ci], v[0], v[1], v[2], v[3], g.cdx, g.cdy);
           }
@@ -717,9 +766,9 @@ __global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS>::NT, 1) k_film(const __g
           if (a.S.zl || a.S.sl) {
             float3 h = f3(0, 0, 0);
             if (a.S.zl) {
-              const float hd[2] = {a.S.hx, a.S.hy};
+              const float hd[3] = {a.S.hx, a.S.hy, a.S.hz};
 #pragma unroll
-              for (int ax = 0; ax < 2; ++ax) {
+              for (int ax = 0; ax < ND / 2; ++ax) {
                 const int j1 = nb[2 * ax + 1], j0 = nb[2 * ax];
                 const float3 v1 = sco[j1] != kVacuum ? f3(st_[j1], st_[D + j1], st_[2 * D + j1]) : mi;
                 const float3 v0 = sco[j0] != kVacuum ? f3(st_[j0], st_[D + j0], st_[2 * D + j0]) : mi;
@@ -765,7 +814,7 @@ __global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS>::NT, 1) k_film(const __g
       }
       if (s == 6) break;
       s = nxt;
-      cur ^= 1;
+      if (!D3) cur ^= 1;
     }
     for (int o = 16; o > 0; o >>= 1) emax = fmaxf(emax, __shfl_xor_sync(0xffffffffu, emax, o));
     if (lane == 0) wmax[tid >> 5] = emax;
@@ -873,9 +922,9 @@ __global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS>::NT, 1) k_film(const __g
 
 }  // namespace
 
-template <int LX, int PH, int ROWS>
+template <int LX, int PH, int ROWS, int PZ>
 bool film_plan_one(const Geom& g, FilmPlan* p) {
-  using F = FilmCfg<LX, PH, ROWS>;
+  using F = FilmCfg<LX, PH, ROWS, PZ>;
   int dev = 0, sms = 0, coop = 0, smem_max = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -884,24 +933,24 @@ bool film_plan_one(const Geom& g, FilmPlan* p) {
   if (!coop) return false;
   const size_t room = smem_max > 2048 ? (size_t)smem_max - 2048 : 0;   // (static: state, coefficients)
   if (ROWS * g.nx > F::CELLS * F::NT) return false;   // (long periodic rows)
-  size_t need = sizeof(float2) * (F::FFT + F::TAB) + sizeof(float) * (7 * (ROWS + 2) + 4 * ROWS) * g.nx +
-                sizeof(RegionLUT);
+  size_t need = sizeof(float2) * (F::FFT + F::TAB + 1) +
+                sizeof(float) * ((3 * F::STG + 1) * F::LR + F::ND * ROWS) * g.nx + sizeof(RegionLUT);
   if (need > room) return false;
   const size_t ob = sizeof(float) * F::OCT;
   p->oct_sm = need + ob <= room;
   if (p->oct_sm) need += ob;
   p->rows = ROWS;
-  p->blocks = std::max((g.ny + ROWS - 1) / ROWS, (LX + F::CPB) / F::CPB);
+  p->blocks = std::max((g.ny + ROWS - 1) / ROWS * g.nz, (LX + F::CPB) / F::CPB);
   p->smem = need;
   // (a function attribute belongs to the device's context; the cap, not this
   // film's need, so that a later film never lowers an earlier one's)
-  if (cudaFuncSetAttribute(k_film<LX, PH, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room) != cudaSuccess) {
+  if (cudaFuncSetAttribute(k_film<LX, PH, ROWS, PZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)room) != cudaSuccess) {
     (void)cudaGetLastError();
     p->rows = 0;
     return false;
   }
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_film<LX, PH, ROWS>, F::NT, need) != cudaSuccess ||
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_film<LX, PH, ROWS, PZ>, F::NT, need) != cudaSuccess ||
       (long long)per_sm * sms < p->blocks) {
     (void)cudaGetLastError();
     p->rows = 0;
@@ -910,11 +959,11 @@ bool film_plan_one(const Geom& g, FilmPlan* p) {
   return true;
 }
 
-template <int LX, int PH, int ROWS>
+template <int LX, int PH, int ROWS, int PZ>
 cudaError_t launch_film_one(const FilmPlan& p, const FilmArgs& args, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.blocks);
-  cfg.blockDim = dim3(FilmCfg<LX, PH, ROWS>::NT);
+  cfg.blockDim = dim3(FilmCfg<LX, PH, ROWS, PZ>::NT);
   cfg.dynamicSmemBytes = p.smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -922,33 +971,64 @@ cudaError_t launch_film_one(const FilmPlan& p, const FilmArgs& args, cudaStream_
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k_film<LX, PH, ROWS>, args);
+  return cudaLaunchKernelEx(&cfg, k_film<LX, PH, ROWS, PZ>, args);
 }
 
 // Rows per block: the fewest whose blocks fit kFilmBlocks.
+#define MM_FILM_CASES(DO)                                                  \
+  if (g.nz == 1) {                                                         \
+    switch (ph) {                                                          \
+      case 16: return DO(16, 1, 1);                                        \
+      case 32: return DO(32, 1, 1);                                        \
+      case 64: return DO(64, 1, 1);                                        \
+      case 128: return DO(128, 1, 1);                                      \
+      case 256: return DO(256, 2, 1);                                      \
+      case 512: return g.ny <= 3 * kFilmBlocks ? DO(512, 3, 1) : DO(512, 4, 1); \
+      default: break;                                                      \
+    }                                                                      \
+  }
+#define MM_FILM3_CASES(DO)                                                 \
+  if (g.pz == 4) {                                                         \
+    switch (ph) {                                                          \
+      case 16: return DO(16, 1, 4);                                        \
+      case 32: return DO(32, 1, 4);                                        \
+      case 64: return DO(64, 1, 4);                                        \
+      case 128: return DO(128, 2, 4);                                      \
+      default: break;                                                      \
+    }                                                                      \
+  } else if (g.pz == 8) {                                                  \
+    switch (ph) {                                                          \
+      case 16: return DO(16, 1, 8);                                        \
+      case 32: return DO(32, 1, 8);                                        \
+      case 64: return DO(64, 2, 8);                                        \
+      case 128: return g.ny <= 3 * (kFilmBlocks / 4) ? DO(128, 3, 8) : DO(128, 4, 8); \
+      default: break;                                                      \
+    }                                                                      \
+  }
+#define MM_FILM_PLAN(PH, ROWS, PZ) film_plan_one<LX, PH, ROWS, PZ>(g, p)
+#define MM_FILM_LAUNCH(PH, ROWS, PZ) launch_film_one<LX, PH, ROWS, PZ>(p, args, s)
 template <int LX>
 bool film_plan_l(const Geom& g, int ph, FilmPlan* p) {
-  switch (ph) {
-    case 16: return film_plan_one<LX, 16, 1>(g, p);
-    case 32: return film_plan_one<LX, 32, 1>(g, p);
-    case 64: return film_plan_one<LX, 64, 1>(g, p);
-    case 128: return film_plan_one<LX, 128, 1>(g, p);
-    case 256: return film_plan_one<LX, 256, 2>(g, p);
-    case 512: return g.ny <= 3 * kFilmBlocks ? film_plan_one<LX, 512, 3>(g, p) : film_plan_one<LX, 512, 4>(g, p);
-    default: return false;
-  }
+  MM_FILM_CASES(MM_FILM_PLAN)
+  return false;
 }
 template <int LX>
 cudaError_t launch_film_l(const FilmPlan& p, int ph, const FilmArgs& args, cudaStream_t s) {
-  switch (ph) {
-    case 16: return launch_film_one<LX, 16, 1>(p, args, s);
-    case 32: return launch_film_one<LX, 32, 1>(p, args, s);
-    case 64: return launch_film_one<LX, 64, 1>(p, args, s);
-    case 128: return launch_film_one<LX, 128, 1>(p, args, s);
-    case 256: return launch_film_one<LX, 256, 2>(p, args, s);
-    case 512: return p.rows == 3 ? launch_film_one<LX, 512, 3>(p, args, s) : launch_film_one<LX, 512, 4>(p, args, s);
-    default: return cudaErrorInvalidValue;
-  }
+  const Geom& g = args.g;
+  MM_FILM_CASES(MM_FILM_LAUNCH)
+  return cudaErrorInvalidValue;
+}
+// thin 3-D grids (in translation units of their own)
+template <int LX>
+bool film3_plan_l(const Geom& g, int ph, FilmPlan* p) {
+  MM_FILM3_CASES(MM_FILM_PLAN)
+  return false;
+}
+template <int LX>
+cudaError_t launch_film3_l(const FilmPlan& p, int ph, const FilmArgs& args, cudaStream_t s) {
+  const Geom& g = args.g;
+  MM_FILM3_CASES(MM_FILM_LAUNCH)
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace mm

@@ -22,9 +22,9 @@ struct FilmArgs {
   const RegionLUT* lut;
   const float* xlut;
   const int* code;
-  float2* spec1;          // [3][hx][ny]
-  float2* spec2;          // [3][ny][hxs]
-  float* halo;            // [3][ny][nx]: the stage input's rows at block edges
+  float2* spec1;          // [3][hx][nz][ny]
+  float2* spec2;          // [3][nz][ny][hxs]
+  float* halo;            // [3][nz][ny][nx]: the stage input's rows that other blocks' stencils read
   DevState* st;
   double* hist;
   const double* fixed;
@@ -45,16 +45,20 @@ struct FilmPlan {
   int rows = 0, blocks = 0, oct_sm = 0;
   size_t smem = 0;
 };
-// Plan of a single-layer fused grid with an open y axis of more than 8 cells
-// on the current device; false where the kernel does not apply (its blocks must all be
+// Plan of a fused grid of one to four layers with open y and z axes and more
+// than 8 cells along y, on the current device; false where the kernel does not apply (its blocks must all be
 // resident at once).  Sets the kernel's shared-memory limit.
 bool film_plan(const Geom& g, FilmPlan* plan);
 cudaError_t launch_film(const FilmPlan& plan, const FilmArgs& args, cudaStream_t s);
 
-// one row length (film_l*.cu)
+// one row length: films (film_l*.cu), two to four layers (film3_l*.cu)
 template <int LX>
 bool film_plan_l(const Geom& g, int ph, FilmPlan* plan);
 template <int LX>
 cudaError_t launch_film_l(const FilmPlan& plan, int ph, const FilmArgs& args, cudaStream_t s);
+template <int LX>
+bool film3_plan_l(const Geom& g, int ph, FilmPlan* plan);
+template <int LX>
+cudaError_t launch_film3_l(const FilmPlan& plan, int ph, const FilmArgs& args, cudaStream_t s);
 
 }  // namespace mm

@@ -293,7 +293,7 @@ int prepare_film(mm_ctx* c) {
   if (c->film_spec) cudaFree(c->film_spec);
   c->film_spec = nullptr;
   if (!film_plan(c->g, &c->film)) return MM_OK;
-  const size_t bytes = 3 * (size_t)c->g.ny * c->g.hxs * sizeof(float2);
+  const size_t bytes = 3 * (size_t)c->g.nz * c->g.ny * c->g.hxs * sizeof(float2);
   MM_CUDA(cudaMalloc((void**)&c->film_spec, bytes));
   MM_CUDA(cudaMemsetAsync(c->film_spec, 0, bytes, c->stream));
   if (!c->film_sync) MM_CUDA(cudaMalloc((void**)&c->film_sync, sizeof(FilmSync)));

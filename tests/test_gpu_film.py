@@ -1,5 +1,5 @@
-"""The persistent film kernel (films step with it by default) at the edges of
-its splits: row lengths and column lengths of every transform size, ragged
+"""The persistent film kernel (films and grids of two to four layers step with
+it by default) at the edges of its splits: row lengths and column lengths of every transform size, ragged
 rows, one and several rows and columns per block, periodic x, DMI,
 spin-transfer torques and both integrators, against the stage kernels'
 path replaying the same step sizes (two float32 paths: 5e-6) and, on small
@@ -27,9 +27,9 @@ def mm():
     return _mm
 
 
-def film(nx, ny, dmi=False, pbcx=False, stt=False):
+def film(nx, ny, dmi=False, pbcx=False, stt=False, nz=1):
     rng = np.random.default_rng(1000 * nx + ny)
-    p = Problem(nx, ny, 1, 2e-9, 2e-9, 1.5e-9)
+    p = Problem(nx, ny, nz, 2e-9, 2e-9, 1.5e-9)
     p.region = rng.integers(0, 3, size=p.shape).astype(np.uint8)
     for r in range(3):
         p.msat[r] = rng.uniform(6e5, 1.1e6)
@@ -61,7 +61,11 @@ def film(nx, ny, dmi=False, pbcx=False, stt=False):
 SHAPES = [(9, 9, {}), (16, 16, {}), (17, 33, {}), (64, 17, {}), (65, 64, {}), (128, 129, {}), (200, 257, {}),
           (257, 100, {}), (256, 256, {}), (100, 445, {}), (512, 512, {}), (300, 60, {"dmi": True}),
           (100, 75, {"dmi": True}), (64, 40, {"pbcx": True, "stt": True}), (33, 20, {"stt": True}),
-          (1024, 20, {"pbcx": True}), (512, 300, {"pbcx": True, "dmi": True})]
+          (1024, 20, {"pbcx": True}), (512, 300, {"pbcx": True, "dmi": True}),
+          # two to four layers: one to four rows per block, ragged layers
+          (20, 30, {"nz": 4}), (96, 96, {"nz": 4}), (17, 120, {"nz": 4}), (33, 17, {"nz": 2}), (128, 64, {"nz": 2}),
+          (40, 128, {"nz": 2}), (130, 33, {"nz": 3}), (30, 20, {"nz": 3, "dmi": True}),
+          (64, 40, {"nz": 2, "pbcx": True, "stt": True})]
 
 
 @pytest.mark.parametrize("method", ["rk45", "rk23"])
@@ -88,7 +92,8 @@ def test_matches_the_stage_kernels(mm, nx, ny, kw, method):
     b.close()
 
 
-@pytest.mark.parametrize("nx,ny,kw", [(17, 9, {}), (40, 33, {"dmi": True}), (32, 20, {"pbcx": True, "stt": True})])
+@pytest.mark.parametrize("nx,ny,kw", [(17, 9, {}), (40, 33, {"dmi": True}), (32, 20, {"pbcx": True, "stt": True}),
+                                      (19, 21, {"nz": 3}), (24, 18, {"nz": 2, "dmi": True, "stt": True})])
 def test_matches_the_oracle(mm, nx, ny, kw):
     p = film(nx, ny, **kw)
     ctx = mm.Context.from_problem(p)
