@@ -315,7 +315,9 @@ int mm_profile_attempts(mm_ctx* ctx, int attempts, int max, int* kinds, double* 
  * per kx plane (y forward, kernel product, y inverse).  2 needs open y and z
  * axes and, in 3-D, py >= 32 and 16 <= pz <= 64, in 2-D (one layer) py of
  * 128, 256 or 512 (MM_ERR_ARG otherwise).  *active (may be NULL) receives the
- * kernels in use: 1 or 2, or 0 on a grid without the fused layout.  The
+ * kernels in use: 1 or 2, or 0 on a grid that has no choice (none of the
+ * cluster kernel's planes: the general convolution, or on larger grids with
+ * open axes, 32 <= py <= 1024 and 16 <= pz <= 128 the three kernels).  The
  * stepping graph is captured again at the next step.  Films (one layer of
  * more than 8 rows, y not periodic) step with a persistent kernel that holds
  * its own (y, z) part by default; with which = 1 or 2 they step with the

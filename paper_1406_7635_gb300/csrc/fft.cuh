@@ -253,6 +253,50 @@ struct RegDft<32, DIR> {
   }
 };
 
+// N = 64: eight 8-point transforms over x[i + 8 r], twiddles W_64^(i k) (tw64),
+// eight 8-point transforms over i: X[k + 8 q].
+template <int DIR>
+struct RegDft<64, DIR> {
+  __device__ __forceinline__ static void run(float2 (&x)[64], const float2* __restrict__ tw64) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      float2 v[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) v[r] = x[i + 8 * r];
+      Dft<8, DIR>::run(v);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        if (i && k) {
+          float2 w = tw64[i * k];
+          if (DIR > 0) w.y = -w.y;
+          v[k] = cmul(v[k], w);
+        }
+        x[i + 8 * k] = v[k];
+      }
+    }
+    // x[i + 8 k]: the i-th input of output class k; its transform X[k + 8 q]
+    // goes to place k 8 + q first, so that each class works on its own values
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      float2 v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = x[i + 8 * k];
+      Dft<8, DIR>::run(v);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) x[8 * k + q] = v[q];
+    }
+    // natural order: X[k + 8 q] from place 8 k + q (an 8 x 8 transpose, register names only)
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+#pragma unroll
+      for (int q = k + 1; q < 8; ++q) {
+        const float2 t = x[8 * k + q];
+        x[8 * k + q] = x[8 * q + k];
+        x[8 * q + k] = t;
+      }
+  }
+};
+
 // pencils stored as rows with pitch PST, twiddles from the global table
 template <int L, int DIR, int NP, int NT, int PST>
 using Fft = FftG<L, DIR, NP, NT, 1, PST, 1>;

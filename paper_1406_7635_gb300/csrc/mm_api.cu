@@ -241,7 +241,7 @@ void demag_yz(mm_ctx* c) {
 // Applies the requested (y, z) kernels: the three-kernel path where the grid
 // allows it (default, or asked for), its buffer allocated or freed to match.
 int apply_yz_choice(mm_ctx* c) {
-  const bool want = yz3_plan(c->g) && c->yz_req != 1;
+  const bool want = yz3_plan(c->g) && (c->yz_req != 1 || large_grid(c->g));   // (large grids have no other)
   if (want && !c->yzt) {
     cudaError_t e = cudaMalloc((void**)&c->yzt, yz3_bytes(c->g));
     if (e != cudaSuccess) {
@@ -584,7 +584,7 @@ int mm_create(mm_ctx** out, int nx, int ny, int nz, double dx, double dy, double
   c->dz = dz;
   c->g = make_geom(nx, ny, nz, dx, dy, dz);
   Geom& g = c->g;
-  fused_plan(g);
+  if (!fused_plan(g)) large_plan(g);
   for (int r = 0; r < kRegions; ++r) {
     std::memset(&c->mat[r], 0, sizeof(mm_material));
     c->mat[r].gamma_ll = kGamma;
@@ -1046,7 +1046,7 @@ int mm_set_pbc(mm_ctx* c, int px, int py, int pz) {
       return fail(MM_ERR_ARG, "a periodic axis needs 1 cell or a power of two >= 4 cells");
   }
   Geom g = make_geom(c->g.nx, c->g.ny, c->g.nz, c->dx, c->dy, c->dz, pbc);
-  fused_plan(g);
+  if (!fused_plan(g)) large_plan(g);
   MM_CUDA(cudaStreamSynchronize(c->stream));
   // buffers whose size depends on the transform lengths
   Buffers& b = c->b;
@@ -1523,7 +1523,7 @@ int mm_sync(mm_ctx* c) {
 int mm_set_yz_kernels(mm_ctx* c, int which, int* active) {
   if (!c) return fail(MM_ERR_ARG, "ctx is NULL");
   if (which < 0 || which > 2) return fail(MM_ERR_ARG, "which must be 0 (default), 1 (cluster) or 2 (three kernels)");
-  if (which == 2 && !yz3_plan(c->g) && !y2d_plan(c->g))
+  if (which == 2 && (large_grid(c->g) || (!yz3_plan(c->g) && !y2d_plan(c->g))))
     return fail(MM_ERR_ARG, "the register-resident (y, z) kernels need open y and z axes and, in 3-D, py >= 32 and "
                             "16 <= pz <= 64, in 2-D py of 128, 256 or 512");
   MM_CUDA(cudaStreamSynchronize(c->stream));
@@ -1539,7 +1539,7 @@ int mm_set_yz_kernels(mm_ctx* c, int which, int* active) {
     MM_CUDA(cudaStreamSynchronize(c->stream));
     MM_CUDA(cudaGetLastError());
   }
-  if (active) *active = c->g.fused ? ((c->yz3 || c->y2d) ? 2 : 1) : 0;
+  if (active) *active = c->g.fused && !large_grid(c->g) ? ((c->yz3 || c->y2d) ? 2 : 1) : 0;
   return MM_OK;
 }
 

@@ -94,7 +94,9 @@ struct Geom {
 // (one wave) 0.165 / 0.197 / 0.161 / 0.203.  The register-resident (y, z)
 // kernels of fft_yz3.cu are always dependents; behind the one-kernel 2-D path
 // the context also makes the row kernel one (launch_rowstage's `dep`).
-inline bool pdl_row(const Geom& g) { return g.fused && g.clz == 2; }
+// (large grids, see large_plan: their row kernels run in many waves)
+inline bool large_grid(const Geom& g) { return g.fused && g.clz == 0; }
+inline bool pdl_row(const Geom& g) { return g.fused && (g.clz == 2 || g.clz == 0); }
 inline bool pdl_yz(const Geom& g) { return !pdl_row(g); }
 
 // Integrator state on the device (one per context).  Every kernel of a step
@@ -191,6 +193,11 @@ void launch_demag_yz(const Geom& g, const Buffers& b, cudaStream_t s);
 // in place in T, y inverse back into the spectrum; yz3_plan(g) tells whether
 // the grid supports it.  launch_demag_fused3: the whole convolution with it.
 bool yz3_plan(const Geom& g);
+// Grids beyond the cluster kernel's planes (fused_plan refuses them) that the
+// three kernels can serve: marks g as fused without a residue split
+// (large_grid), so that the context steps with the row-stage kernels and
+// always convolves with the three kernels.
+bool large_plan(Geom& g);
 // 2-D grids: y forward, kernel product and y inverse of a kx plane in one
 // block (fft_yz3.cu), in place in the spectrum; y2d_plan(g) tells whether
 // the grid supports it.  launch_demag_fused2d: the whole convolution with it.

@@ -37,7 +37,7 @@ enum { ROW_K1 = 0, ROW_NEXT = 1, ROW_LAST = 2 };
 
 __device__ __forceinline__ float* stage_buf(const Buffers& b, int s) { return (s & 1) ? b.ms2 : b.ms; }
 
-// 32-bit indices: the fused layout has nz <= 32 and at most 2^28 cells
+// 32-bit indices: the fused layout has at most 3 * 513 * 64 * 512 points
 __device__ __forceinline__ int tix(const Geom& g, int c, int kx, int z, int y) {
   return ((c * g.hx + kx) * g.nz + z) * g.ny + y;
 }
@@ -933,7 +933,9 @@ cudaError_t prepare_rowstage(const Geom& g) {
 void rowstage_maps(const Geom& g, const Buffers& b, RsMaps* m) {
   std::memset(m, 0, sizeof(RsMaps));
   const int L = g.lx, rows = rs_rows(g);
-  if (!g.fused || g.pbcx || !b.spec || !b.ms || !b.ms2 || !b.code) return;
+  // (large grids keep asynchronous copies: their steps take no bounded waits,
+  // whatever the context's wait limit, as before they had row-stage kernels)
+  if (!g.fused || g.pbcx || large_grid(g) || !b.spec || !b.ms || !b.ms2 || !b.code) return;
   if (L >= 32 && L <= 128 && rows >= 8 && g.ny % 2 == 0) {
     const cuuint64_t dims[4] = {(cuuint64_t)g.ny, (cuuint64_t)g.nz, (cuuint64_t)g.hx, 3};
     const cuuint64_t st[3] = {(cuuint64_t)g.ny * 8, (cuuint64_t)g.nz * g.ny * 8, (cuuint64_t)g.hx * g.nz * g.ny * 8};
