@@ -470,7 +470,9 @@ __global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS, PZ>::NT, 1) k_film(const
   };
 
   float* rowf = reinterpret_cast<float*>(fb);
-  // float index of cell x of component c, row r in the row pencils
+  // float index of cell x of component c, row r in the row pencils; a cell
+  // uses the place rix ^ 1 of the exchanged parts for its B_demag and, written
+  // by the same thread after that is read, for its M
   auto rix = [&](int c, int r, int x) { return 2 * ((c * ROWS + r) * FX::AREA + FX::pos(x >> 1)) + (x & 1); };
   // lane roles in the transforms
   const int px = tid / FX::LANES, jx = tid % FX::LANES;   // row pencil c ROWS + r
@@ -493,7 +495,7 @@ __global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS, PZ>::NT, 1) k_film(const
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         if (!D3) st_[c * D + (r + 1) * nx + x] = v[c];
-        rowf[rix(c, r, x)] = ms * v[c];
+        rowf[rix(c, r, x) ^ 1] = ms * v[c];
         if (D3 || r == 0 || r == nrow - 1) a.halo[c * n + own + e] = v[c];
       }
     };
@@ -525,7 +527,7 @@ __global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS, PZ>::NT, 1) k_film(const
         const int nin = (nx + 1) / 2;
         float2* e = fb + px * FX::AREA;
         FX::run(e, tx, jx, [&](int i, int) {
-          float2 v = i < nin ? e[FX::pos(i)] : make_float2(0.f, 0.f);
+          float2 v = i < nin ? swapc(e[FX::pos(i)]) : make_float2(0.f, 0.f);
           if ((nx & 1) && i == nin - 1) v.y = 0.f;   // (x = nx is padding)
           return v;
         });
