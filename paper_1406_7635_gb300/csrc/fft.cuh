@@ -18,6 +18,38 @@ constexpr int kTwN = 2048;   // twiddle table length: largest supported L
 
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// The same sums as one packed instruction each (two float32 lanes, each
+// rounded as the scalar one): half the issue slots of a transform's additions.
+// Used where a register transform is bound by instruction issue, the (y, z)
+// kernels of fft_yz3.cu; an RK restart of 256 x 256 x 64 cells takes 8.09 ms
+// with them (8.29 ms without), of 77 x 93 x 21 cells 3.24 ms (3.28), the stray
+// field of 128 x 128 x 32 cells 73 us (74.5).  The films' transforms stay
+// scalar: there the compiler fuses some of the sums into multiply-adds, and
+// without that the Zeeman energy of a 256 x 256 film was further off.
+__device__ __forceinline__ unsigned long long pack2(float2 a) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long r) {
+  float2 a;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a.x), "=f"(a.y) : "l"(r));
+  return a;
+}
+template <bool PK>
+__device__ __forceinline__ float2 caddp(float2 a, float2 b) {
+  if (!PK) return cadd(a, b);
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+  return unpack2(r);
+}
+template <bool PK>
+__device__ __forceinline__ float2 csubp(float2 a, float2 b) {
+  if (!PK) return csub(a, b);
+  unsigned long long r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+  return unpack2(r);
+}
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
@@ -64,48 +96,48 @@ __device__ __forceinline__ float2 rot16(float2 o) {
 }
 
 // In-register DFT of length R (R = 1, 2, 4, 8, 16), natural order in and out,
-// by recursive even/odd splitting.
-template <int R, int DIR>
+// by recursive even/odd splitting.  PK: packed additions (caddp).
+template <int R, int DIR, bool PK = false>
 struct Dft {
   __device__ __forceinline__ static void run(float2 (&x)[R]) {
     float2 e[R / 2], o[R / 2];
 #pragma unroll
     for (int i = 0; i < R / 2; ++i) { e[i] = x[2 * i]; o[i] = x[2 * i + 1]; }
-    Dft<R / 2, DIR>::run(e);
-    Dft<R / 2, DIR>::run(o);
+    Dft<R / 2, DIR, PK>::run(e);
+    Dft<R / 2, DIR, PK>::run(o);
     combine<0>(x, e, o);
   }
   template <int K>
   __device__ __forceinline__ static void combine(float2 (&x)[R], const float2 (&e)[R / 2], const float2 (&o)[R / 2]) {
     if constexpr (K < R / 2) {
       const float2 t = rot16<K * (16 / R), DIR>(o[K]);
-      x[K] = cadd(e[K], t);
-      x[K + R / 2] = csub(e[K], t);
+      x[K] = caddp<PK>(e[K], t);
+      x[K + R / 2] = csubp<PK>(e[K], t);
       combine<K + 1>(x, e, o);
     }
   }
 };
-template <int DIR>
-struct Dft<1, DIR> {
+template <int DIR, bool PK>
+struct Dft<1, DIR, PK> {
   __device__ __forceinline__ static void run(float2 (&)[1]) {}
 };
-template <int DIR>
-struct Dft<2, DIR> {
+template <int DIR, bool PK>
+struct Dft<2, DIR, PK> {
   __device__ __forceinline__ static void run(float2 (&x)[2]) {
     const float2 a = x[0];
-    x[0] = cadd(a, x[1]);
-    x[1] = csub(a, x[1]);
+    x[0] = caddp<PK>(a, x[1]);
+    x[1] = csubp<PK>(a, x[1]);
   }
 };
-template <int DIR>
-struct Dft<4, DIR> {
+template <int DIR, bool PK>
+struct Dft<4, DIR, PK> {
   __device__ __forceinline__ static void run(float2 (&x)[4]) {
-    const float2 a0 = cadd(x[0], x[2]), a1 = csub(x[0], x[2]);
-    const float2 a2 = cadd(x[1], x[3]), a3 = mul_dir_i<DIR>(csub(x[1], x[3]));
-    x[0] = cadd(a0, a2);
-    x[2] = csub(a0, a2);
-    x[1] = cadd(a1, a3);
-    x[3] = csub(a1, a3);
+    const float2 a0 = caddp<PK>(x[0], x[2]), a1 = csubp<PK>(x[0], x[2]);
+    const float2 a2 = caddp<PK>(x[1], x[3]), a3 = mul_dir_i<DIR>(csubp<PK>(x[1], x[3]));
+    x[0] = caddp<PK>(a0, a2);
+    x[2] = csubp<PK>(a0, a2);
+    x[1] = caddp<PK>(a1, a3);
+    x[3] = csubp<PK>(a1, a3);
   }
 };
 
@@ -227,12 +259,12 @@ struct FftG<L, DIR, NP, NT, INNER, BS, ES, TWL, IS, P, true> {
 // In-register DFT of length N, natural order in and out: Dft for N <= 16;
 // N = 32 as two 16-point halves (even / odd samples) combined with W_32^k,
 // read from tw32[k] = exp(-2 pi i k / 32) (conjugated for DIR > 0).
-template <int N, int DIR>
+template <int N, int DIR, bool PK = false>
 struct RegDft {
-  __device__ __forceinline__ static void run(float2 (&x)[N], const float2* __restrict__) { Dft<N, DIR>::run(x); }
+  __device__ __forceinline__ static void run(float2 (&x)[N], const float2* __restrict__) { Dft<N, DIR, PK>::run(x); }
 };
-template <int DIR>
-struct RegDft<32, DIR> {
+template <int DIR, bool PK>
+struct RegDft<32, DIR, PK> {
   __device__ __forceinline__ static void run(float2 (&x)[32], const float2* __restrict__ tw32) {
     float2 e[16], o[16];
 #pragma unroll
@@ -240,30 +272,30 @@ struct RegDft<32, DIR> {
       e[i] = x[2 * i];
       o[i] = x[2 * i + 1];
     }
-    Dft<16, DIR>::run(e);
-    Dft<16, DIR>::run(o);
+    Dft<16, DIR, PK>::run(e);
+    Dft<16, DIR, PK>::run(o);
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
       float2 w = tw32[k];
       if (DIR > 0) w.y = -w.y;
       const float2 t = cmul(o[k], w);
-      x[k] = cadd(e[k], t);
-      x[k + 16] = csub(e[k], t);
+      x[k] = caddp<PK>(e[k], t);
+      x[k + 16] = csubp<PK>(e[k], t);
     }
   }
 };
 
 // N = 64: eight 8-point transforms over x[i + 8 r], twiddles W_64^(i k) (tw64),
 // eight 8-point transforms over i: X[k + 8 q].
-template <int DIR>
-struct RegDft<64, DIR> {
+template <int DIR, bool PK>
+struct RegDft<64, DIR, PK> {
   __device__ __forceinline__ static void run(float2 (&x)[64], const float2* __restrict__ tw64) {
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
       float2 v[8];
 #pragma unroll
       for (int r = 0; r < 8; ++r) v[r] = x[i + 8 * r];
-      Dft<8, DIR>::run(v);
+      Dft<8, DIR, PK>::run(v);
 #pragma unroll
       for (int k = 0; k < 8; ++k) {
         if (i && k) {
@@ -281,7 +313,7 @@ struct RegDft<64, DIR> {
       float2 v[8];
 #pragma unroll
       for (int i = 0; i < 8; ++i) v[i] = x[i + 8 * k];
-      Dft<8, DIR>::run(v);
+      Dft<8, DIR, PK>::run(v);
 #pragma unroll
       for (int q = 0; q < 8; ++q) x[8 * k + q] = v[q];
     }

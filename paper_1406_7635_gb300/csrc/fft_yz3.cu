@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(kZNT, z_min_blocks(LZH)) k_zk(Geom g, float2* 
 #pragma unroll
     for (int z = 0; z < LZH; ++z) v[z] = cmul(v[z], twz[z]);
   }
-  RegDft<LZH, -1>::run(v, twl);   // v[l] = A_c(kz = 2 l + rz)
+  RegDft<LZH, -1, true>::run(v, twl);   // v[l] = A_c(kz = 2 l + rz)
 #pragma unroll
   for (int l = 0; l < LZH; ++l) sA[(c * PZ + 2 * l + rz) * CP + col] = v[l];
   __syncthreads();
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kZNT, z_min_blocks(LZH)) k_zk(Geom g, float2* 
 #pragma unroll
   for (int l = 0; l < LZH; ++l) v[l] = sA[(c * PZ + 2 * l + rz) * CP + col];
   // 3. inverse class transform: v[z] = sum_l B_c(2 l + rz) W_LZH^(-z l)
-  RegDft<LZH, 1>::run(v, twl);
+  RegDft<LZH, 1, true>::run(v, twl);
   // 4. b[z] = V_0[z] + conj(W_PZ^z) V_1[z]: the class-0 lane writes z < LZH / 2,
   //    the class-1 lane (16 lanes up) the rest, each with the partner's half
   //    by a shuffle
@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(kY2NT, kY3MinBlocks) k_yf3(Geom g, const float
     const float2 x = (z < nz && y < ny) ? src[y] : make_float2(0.f, 0.f);
     v[r] = cls ? cmul(x, twc[y]) : x;
   }
-  Dft<16, -1>::run(v);                                    // v[k1] = sum_r x W_16^(r k1)
+  Dft<16, -1, true>::run(v);                                    // v[k1] = sum_r x W_16^(r k1)
 #pragma unroll
   for (int k1 = 1; k1 < 16; ++k1) v[k1] = cmul(v[k1], twh[(j * k1) & (PH - 1)]);
 #pragma unroll
@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(kY2NT, kY3MinBlocks) k_yf3(Geom g, const float
     for (int jj = 0; jj < G; ++jj) w[h][jj] = e[jj * EP + j + G * h];
 #pragma unroll
   for (int h = 0; h < H; ++h) {
-    Dft<G, -1>::run(w[h]);                                // w[h][k2] = X(k1 + 16 k2), k1 = j + G h
+    Dft<G, -1, true>::run(w[h]);                                // w[h][k2] = X(k1 + 16 k2), k1 = j + G h
     if (z < nz) {
 #pragma unroll
       for (int k2 = 0; k2 < G; ++k2) dst[2 * (j + G * h + 16 * k2) + cls] = w[h][k2];
@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(kY2NT, kY3MinBlocks) k_yi3(Geom g, const float
       w[h][k2] = z < nz ? src[2 * (j + G * h + 16 * k2) + cls] : make_float2(0.f, 0.f);
 #pragma unroll
   for (int h = 0; h < H; ++h) {
-    Dft<G, 1>::run(w[h]);                                 // w[h][jj] = V(jj, k1)
+    Dft<G, 1, true>::run(w[h]);                                 // w[h][jj] = V(jj, k1)
 #pragma unroll
     for (int jj = 0; jj < G; ++jj) {
       const int k1 = j + G * h;
@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(kY2NT, kY3MinBlocks) k_yi3(Geom g, const float
   float2 v[16];
 #pragma unroll
   for (int k1 = 0; k1 < 16; ++k1) v[k1] = e[j * EP + k1];
-  Dft<16, 1>::run(v);                                     // v[r] = x_cls(j + G r)
+  Dft<16, 1, true>::run(v);                                     // v[r] = x_cls(j + G r)
   // y = j + G r: x_0 + conj(W_(2 PH)^y) x_1; the class-0 lane writes r < 8,
   // the class-1 lane (its neighbour) r >= 8, each with the partner's half
   float2* __restrict__ out = spec + ((c * g.hx + kx) * nz + (z < nz ? z : 0)) * ny;
