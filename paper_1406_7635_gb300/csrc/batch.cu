@@ -102,6 +102,8 @@ __global__ void k_b_begin(InstState* st, int n, double t_end) {
   if (!s.done) prepare(s);
 }
 
+// the input of stage 0 (s = 0: m itself) or 1; the later ones come out of
+// the stage before them (k_b_stage)
 __global__ void k_b_stage_input(Geom g, BPtrs p, float* __restrict__ ms, const InstState* __restrict__ st, int s) {
   const int inst = blockIdx.y;
   const InstState& S = st[inst];
@@ -113,10 +115,9 @@ __global__ void k_b_stage_input(Geom g, BPtrs p, float* __restrict__ ms, const I
   const int par = S.parity;
   const float* __restrict__ m = (par ? p.m1 : p.m0) + o;
   float a0 = m[i], a1 = m[n + i], a2 = m[2 * n + i];
-  for (int j = 0; j < s; ++j) {
-    const float a = S.ah[s][j];
-    if (a == 0.0f) continue;
-    const float* __restrict__ k = bpick(p, role(j, par)) + o;
+  const float a = S.ah[s][0];
+  if (s > 0 && a != 0.0f) {
+    const float* __restrict__ k = bpick(p, role(0, par)) + o;
     a0 = fmaf(a, k[i], a0);
     a1 = fmaf(a, k[n + i], a1);
     a2 = fmaf(a, k[2 * n + i], a2);
@@ -125,43 +126,6 @@ __global__ void k_b_stage_input(Geom g, BPtrs p, float* __restrict__ ms, const I
   mso[i] = a0;
   mso[n + i] = a1;
   mso[2 * n + i] = a2;
-}
-
-// effective field (demag + exchange + static Zeeman) and LL torque
-__global__ void k_b_torque(Geom g, BPtrs p, const float* __restrict__ ms, const float* __restrict__ bd,
-                           const InstParams* __restrict__ prm, const InstState* __restrict__ st, int s) {
-  const int inst = blockIdx.y;
-  const InstState& S = st[inst];
-  if (S.done) return;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;   // in-instance offsets: 3 n < 2^31
-  if (i >= g.n) return;
-  const long long o = (long long)inst * 3 * g.n;
-  const int n = (int)g.n;
-  const float* __restrict__ m = ms + o;
-  const float* __restrict__ bdo = bd + o;
-  const InstParams P = prm[inst];
-  const int x = i % g.nx, y = (i / g.nx) % g.ny, z = i / (g.nx * g.ny);
-  const float mx = m[i], my = m[n + i], mz = m[2 * n + i];
-  float bx = bdo[i] + P.b[0], by = bdo[n + i] + P.b[1], bz = bdo[2 * n + i] + P.b[2];
-  auto nb = [&](int j, float id2) {
-    const float c = P.exch * id2;
-    bx += c * (m[j] - mx);
-    by += c * (m[n + j] - my);
-    bz += c * (m[2 * n + j] - mz);
-  };
-  const int sy = g.nx, sz = g.nx * g.ny;
-  if (x > 0) nb(i - 1, g.idx2);
-  if (x < g.nx - 1) nb(i + 1, g.idx2);
-  if (y > 0) nb(i - sy, g.idy2);
-  if (y < g.ny - 1) nb(i + sy, g.idy2);
-  if (z > 0) nb(i - sz, g.idz2);
-  if (z < g.nz - 1) nb(i + sz, g.idz2);
-  const float cx = my * bz - mz * by, cy = mz * bx - mx * bz, cz = mx * by - my * bx;
-  const float dx = my * cz - mz * cy, dy = mz * cx - mx * cz, dz = mx * cy - my * cx;
-  float* __restrict__ k = bpick(p, role(s, S.parity)) + o;
-  k[i] = P.gfac * (cx + P.alpha * dx);
-  k[n + i] = P.gfac * (cy + P.alpha * dy);
-  k[2 * n + i] = P.gfac * (cz + P.alpha * dz);
 }
 
 // Sec. IV controller, per instance (the same readings as the single path).
@@ -201,50 +165,118 @@ __device__ void b_controller(InstState& s, double* __restrict__ hist) {
   if (!s.done) prepare(s);
 }
 
-__global__ void k_b_error(Geom g, BPtrs p, const float* __restrict__ ms, InstState* __restrict__ st,
-                          double* __restrict__ hist) {
+// whether stage s takes k_j (bA's zero entries beyond the diagonal aside)
+__host__ __device__ constexpr bool takes(int s, int j) { return j < s && !(s == 6 && j == 1); }
+
+// Effective field (demag + exchange + static Zeeman) and LL torque of stage
+// S, k_S, and what follows from a cell's own slopes while they are at hand:
+// S = 1 .. 5 the cell's input of stage S + 1 (to ms_next; ms is still read by
+// the neighbours), S = 6 its error and new m and the instance's step decision.
+// Bound by memory and by the drain between dependent launches: as kernels of
+// their own the next input and the error read k_S and m again and cost six
+// more launches per attempt.  64 instances of 901120 cells in all: 23.92 ms
+// for one picosecond with the states set and read (24.42 ms with them apart).
+template <int S>
+__global__ void k_b_stage(Geom g, BPtrs p, const float* __restrict__ ms, float* __restrict__ ms_next,
+                          const float* __restrict__ bd, const InstParams* __restrict__ prm,
+                          InstState* __restrict__ st, double* __restrict__ hist) {
   const int inst = blockIdx.y;
-  InstState& S = st[inst];
-  if (S.done) return;   // uniform over the instance's blocks
+  InstState& I = st[inst];
+  if (I.done) return;   // uniform over the instance's blocks
   const int i = blockIdx.x * blockDim.x + threadIdx.x;   // in-instance offsets: 3 n < 2^31
   const long long o = (long long)inst * 3 * g.n;
-  const int n = (int)g.n;
-  const int par = S.parity;
+  const int n = (int)g.n, par = I.parity;
   float e = 0.0f;
   if (i < n) {
-    float ex = 0.f, ey = 0.f, ez = 0.f;
-    for (int j = 0; j < 7; ++j) {
-      const float c = S.eh[j];
-      if (c == 0.0f) continue;
-      const float* __restrict__ k = bpick(p, role(j, par)) + o;
-      ex = fmaf(c, k[i], ex);
-      ey = fmaf(c, k[n + i], ey);
-      ez = fmaf(c, k[2 * n + i], ez);
+    const float* __restrict__ m = ms + o;
+    const float* __restrict__ bdo = bd + o;
+    const InstParams P = prm[inst];
+    // the cell's m and slopes, loaded together
+    float m0[3] = {0.f, 0.f, 0.f}, ks[6][3];
+    if (S >= 1 && S <= 5) {
+      const float* __restrict__ mm0 = (par ? p.m1 : p.m0) + o;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) m0[c] = mm0[c * n + i];
     }
-    e = sqrtf(ex * ex + ey * ey + ez * ez);
-    if (!(e <= FLT_MAX)) e = __int_as_float(0x7f800000);
-    float* __restrict__ mnew = (par ? p.m0 : p.m1) + o;
-    const float* __restrict__ mso = ms + o;
-    const float mx = mso[i], my = mso[n + i], mz = mso[2 * n + i];
-    const float inv = rsqrtf(mx * mx + my * my + mz * mz);
-    mnew[i] = mx * inv;
-    mnew[n + i] = my * inv;
-    mnew[2 * n + i] = mz * inv;
+    if (S >= 1) {
+#pragma unroll
+      for (int j = 0; j < S; ++j) {
+        if (S == 6 ? j == 1 : !takes(S + 1, j)) continue;
+        const float* __restrict__ k = bpick(p, role(j, par)) + o;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) ks[j][c] = k[c * n + i];
+      }
+    }
+    const int x = i % g.nx, y = (i / g.nx) % g.ny, z = i / (g.nx * g.ny);
+    const float mx = m[i], my = m[n + i], mz = m[2 * n + i];
+    float bx = bdo[i] + P.b[0], by = bdo[n + i] + P.b[1], bz = bdo[2 * n + i] + P.b[2];
+    auto nb = [&](int j, float id2) {
+      const float c = P.exch * id2;
+      bx += c * (m[j] - mx);
+      by += c * (m[n + j] - my);
+      bz += c * (m[2 * n + j] - mz);
+    };
+    const int sy = g.nx, sz = g.nx * g.ny;
+    if (x > 0) nb(i - 1, g.idx2);
+    if (x < g.nx - 1) nb(i + 1, g.idx2);
+    if (y > 0) nb(i - sy, g.idy2);
+    if (y < g.ny - 1) nb(i + sy, g.idy2);
+    if (z > 0) nb(i - sz, g.idz2);
+    if (z < g.nz - 1) nb(i + sz, g.idz2);
+    const float cx = my * bz - mz * by, cy = mz * bx - mx * bz, cz = mx * by - my * bx;
+    const float dx = my * cz - mz * cy, dy = mz * cx - mx * cz, dz = mx * cy - my * cx;
+    const float kk[3] = {P.gfac * (cx + P.alpha * dx), P.gfac * (cy + P.alpha * dy), P.gfac * (cz + P.alpha * dz)};
+    float* __restrict__ k = bpick(p, role(S, par)) + o;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) k[c * n + i] = kk[c];
+    if constexpr (S >= 1 && S <= 5) {
+      float* __restrict__ out = ms_next + o;
+#pragma unroll
+      for (int j = 0; j <= S; ++j) {
+        if (!takes(S + 1, j)) continue;
+        const float a = I.ah[S + 1][j];
+        if (a == 0.0f) continue;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) m0[c] = fmaf(a, j < S ? ks[j][c] : kk[c], m0[c]);
+      }
+#pragma unroll
+      for (int c = 0; c < 3; ++c) out[c * n + i] = m0[c];
+    }
+    if constexpr (S == 6) {
+      float ev[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+      for (int j = 0; j < 7; ++j) {
+        if (j == 1) continue;   // (bE[1] is zero)
+        const float c = I.eh[j];
+        if (c == 0.0f) continue;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) ev[q] = fmaf(c, j < 6 ? ks[j < 6 ? j : 0][q] : kk[q], ev[q]);
+      }
+      e = sqrtf(ev[0] * ev[0] + ev[1] * ev[1] + ev[2] * ev[2]);
+      if (!(e <= FLT_MAX)) e = __int_as_float(0x7f800000);
+      float* __restrict__ mnew = (par ? p.m0 : p.m1) + o;
+      const float inv = rsqrtf(mx * mx + my * my + mz * mz);
+      mnew[i] = mx * inv;
+      mnew[n + i] = my * inv;
+      mnew[2 * n + i] = mz * inv;
+    }
   }
-  for (int off = 16; off > 0; off >>= 1) e = fmaxf(e, __shfl_xor_sync(0xffffffffu, e, off));
-  __shared__ float wmax[32];
-  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = e;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    float v = threadIdx.x < (blockDim.x >> 5) ? wmax[threadIdx.x] : 0.0f;
-    for (int off = 16; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
-    if (threadIdx.x == 0) {
-      atomicMax(&S.err_bits, __float_as_uint(v));
-      __threadfence();
-      const unsigned int t = atomicAdd(&S.ticket, 1u);
-      if (t == gridDim.x - 1) {
+  if constexpr (S == 6) {
+    for (int off = 16; off > 0; off >>= 1) e = fmaxf(e, __shfl_xor_sync(0xffffffffu, e, off));
+    __shared__ float wmax[32];
+    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = e;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      float v = threadIdx.x < (blockDim.x >> 5) ? wmax[threadIdx.x] : 0.0f;
+      for (int off = 16; off > 0; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
+      if (threadIdx.x == 0) {
+        atomicMax(&I.err_bits, __float_as_uint(v));
         __threadfence();
-        b_controller(S, hist + (long long)inst * kBatchHist);
+        const unsigned int t = atomicAdd(&I.ticket, 1u);
+        if (t == gridDim.x - 1) {
+          __threadfence();
+          b_controller(I, hist + (long long)inst * kBatchHist);
+        }
       }
     }
   }
@@ -288,6 +320,7 @@ struct BClass {
   int first = 0;            // offset of its first instance in the state array
   std::vector<int> ids;     // global instance indices
   Buffers b{};
+  float* ms2 = nullptr;     // the other stage input (a stage writes the next one)
   float* msat = nullptr;
   InstParams* prm = nullptr;
   double* hist = nullptr;
@@ -343,21 +376,34 @@ BatchArgs bargs(const mm_batch* B, const BClass& c) {
   return BatchArgs{c.B, c.msat, &B->st[c.first].done, (int)(sizeof(InstState) / sizeof(int))};
 }
 
-// stage s of every unfinished instance of class c (s = 0: first stage at m)
-void enqueue_stage(mm_batch* B, BClass& c, int s, cudaStream_t st) {
+// stage S of every unfinished instance of class c from its input in ms[S & 1]
+template <int S>
+void enqueue_eval(mm_batch* B, BClass& c, cudaStream_t st) {
   const Geom& g = c.g;
-  dim3 grid((unsigned)((g.n + kT - 1) / kT), c.B);
-  k_b_stage_input<<<grid, kT, 0, st>>>(g, bptrs(c), c.b.ms, B->st + c.first, s);
+  const dim3 grid((unsigned)((g.n + kT - 1) / kT), c.B);
+  float* ms[2] = {c.b.ms, c.ms2};
   Buffers bb = c.b;
   bb.st = nullptr;
-  launch_demag_fused_batch(g, bb, c.b.ms, st, bargs(B, c));
-  k_b_torque<<<grid, kT, 0, st>>>(g, bptrs(c), c.b.ms, c.b.bd, c.prm, B->st + c.first, s);
+  launch_demag_fused_batch(g, bb, ms[S & 1], st, bargs(B, c));
+  k_b_stage<S><<<grid, kT, 0, st>>>(g, bptrs(c), ms[S & 1], ms[(S + 1) & 1], c.b.bd, c.prm, B->st + c.first, c.hist);
+}
+
+// k_0 of every unfinished instance of class c at its m
+void enqueue_k1(mm_batch* B, BClass& c, cudaStream_t st) {
+  const dim3 grid((unsigned)((c.g.n + kT - 1) / kT), c.B);
+  k_b_stage_input<<<grid, kT, 0, st>>>(c.g, bptrs(c), c.b.ms, B->st + c.first, 0);
+  enqueue_eval<0>(B, c, st);
 }
 
 void enqueue_attempt(mm_batch* B, BClass& c, cudaStream_t st) {
-  for (int s = 1; s < 7; ++s) enqueue_stage(B, c, s, st);
-  dim3 grid((unsigned)((c.g.n + kT - 1) / kT), c.B);
-  k_b_error<<<grid, kT, 0, st>>>(c.g, bptrs(c), c.b.ms, B->st + c.first, c.hist);
+  const dim3 grid((unsigned)((c.g.n + kT - 1) / kT), c.B);
+  k_b_stage_input<<<grid, kT, 0, st>>>(c.g, bptrs(c), c.ms2, B->st + c.first, 1);
+  enqueue_eval<1>(B, c, st);
+  enqueue_eval<2>(B, c, st);
+  enqueue_eval<3>(B, c, st);
+  enqueue_eval<4>(B, c, st);
+  enqueue_eval<5>(B, c, st);
+  enqueue_eval<6>(B, c, st);
 }
 
 int build_batch_graph(mm_batch* B) {
@@ -544,6 +590,7 @@ int mm_batch_create(mm_batch** out, int n, const mm_instance_spec* specs, int de
     alloc((void**)&C.b.m[1], vec);
     for (int j = 0; j < 7; ++j) alloc((void**)&C.b.k[j], vec);
     alloc((void**)&C.b.ms, vec);
+    alloc((void**)&C.ms2, vec);
     alloc((void**)&C.b.bd, vec);
     alloc((void**)&C.b.spec, (size_t)C.B * 3 * g.hx * g.nz * g.ny * sizeof(float2));
     alloc((void**)&C.b.kt, 6 * (size_t)g.hkx * g.hky * g.hkz * sizeof(float));
@@ -594,7 +641,7 @@ int mm_batch_create(mm_batch** out, int n, const mm_instance_spec* specs, int de
   int rc = write_states(B);
   if (rc) return cleanup(rc);
   // one pass of every kernel outside any capture (sets launch attributes)
-  for (int c = 0; c < nc; ++c) enqueue_stage(B, B->cls[c], 0, B->stream);
+  for (int c = 0; c < nc; ++c) enqueue_k1(B, B->cls[c], B->stream);
   e = cudaStreamSynchronize(B->stream);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) return cleanup(bfail(MM_ERR_CUDA, std::string("batch warm-up: ") + cudaGetErrorString(e)));
@@ -609,7 +656,7 @@ int mm_batch_destroy(mm_batch* B) {
   if (B->exec) cudaGraphExecDestroy(B->exec);
   for (BClass& C : B->cls) {
     void* ptrs[] = {C.b.m[0], C.b.m[1], C.b.k[0], C.b.k[1], C.b.k[2], C.b.k[3], C.b.k[4], C.b.k[5], C.b.k[6],
-                    C.b.ms,   C.b.bd,   C.b.spec, C.b.kt,   C.b.ktf,  C.msat,   C.prm,    C.hist};
+                    C.b.ms,   C.ms2,    C.b.bd,   C.b.spec, C.b.kt,   C.b.ktf,  C.msat,   C.prm,    C.hist};
     for (void* p : ptrs)
       if (p) cudaFree(p);
   }
@@ -690,7 +737,7 @@ int mm_batch_run(mm_batch* B, double t_end) {
   k_b_begin<<<(B->n + 127) / 128, 128, 0, B->stream>>>(B->st, B->n, t_end);
   MMB_CUDA(cudaGetLastError());
   if (!B->k1_valid) {
-    for (BClass& C : B->cls) enqueue_stage(B, C, 0, B->stream);
+    for (BClass& C : B->cls) enqueue_k1(B, C, B->stream);
     MMB_CUDA(cudaGetLastError());
     B->k1_valid = true;
   }
