@@ -86,7 +86,12 @@ __device__ __forceinline__ unsigned pack_bf16(float lo, float hi) {
   return *reinterpret_cast<const unsigned*>(&v);
 }
 
-template <bool TA, bool TB>
+// VEC (TA false; see gemm_vec): operands in 16-byte loads, four values of
+// the contiguous dimension each.  The products are bound by the issue of the
+// loads and conversions around the tensor cores: 8 loads per thread and step
+// in place of 32.  512 x 512 forward pass of width 32, 24 modes: 512 us (537
+// with 4-byte loads only).
+template <bool TA, bool TB, bool VEC>
 __global__ void __launch_bounds__(128) k_gemm(GemmArgs a) {
   __shared__ __align__(16) __nv_bfloat16 As[BM][APITCH];
   __shared__ __align__(16) __nv_bfloat16 Bs[BN][APITCH];
@@ -112,8 +117,56 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs a) {
   // operand pairs of one BK step in registers: the next step's global loads
   // are in flight while the tensor cores work on the current one
   constexpr int PA = BM * BK / 2 / 128, PB = BN * BK / 2 / 128;
-  float ra[PA][2], rb[PB][2];
-  auto load = [&](int k0) {
+  static_assert(!(VEC && TA), "16-byte loads run along k of A");
+  // quads of a BK step: A (and B from [n][k]) four k of a row, a row in 8
+  // neighbouring lanes; B from [k][n] four n of k = lane, so that the
+  // transposing 2-byte stores of a warp fall on neighbouring places
+  constexpr int QA = BM * BK / 4 / 128, QB = BN * BK / 4 / 128;
+  float4 qa[VEC ? QA : 1], qb[VEC ? QB : 1];
+  auto loadq = [&](int k0) {
+#pragma unroll
+    for (int u = 0; u < QA; ++u) {
+      const int e = tid + u * 128, gm = m0 + e / (BK / 4), gk = k0 + 4 * (e % (BK / 4));
+      qa[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (gm < a.M && gk < kend) qa[u] = *reinterpret_cast<const float4*>(A + (long long)gm * a.lda + gk);
+    }
+#pragma unroll
+    for (int u = 0; u < QB; ++u) {
+      const int e = tid + u * 128;
+      qb[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (TB) {
+        const int gn = n0 + e / (BK / 4), gk = k0 + 4 * (e % (BK / 4));
+        if (gn < a.N && gk < kend) qb[u] = *reinterpret_cast<const float4*>(B + (long long)gn * a.ldb + gk);
+      } else {
+        const int gn = n0 + 4 * (e / BK), gk = k0 + e % BK;
+        if (gn < a.N && gk < kend) qb[u] = *reinterpret_cast<const float4*>(B + (long long)gk * a.ldb + gn);
+      }
+    }
+  };
+  auto storeq = [&]() {
+#pragma unroll
+    for (int u = 0; u < QA; ++u) {
+      const int e = tid + u * 128;
+      *reinterpret_cast<uint2*>(&As[e / (BK / 4)][4 * (e % (BK / 4))]) =
+          make_uint2(pack_bf16(qa[u].x, qa[u].y), pack_bf16(qa[u].z, qa[u].w));
+    }
+#pragma unroll
+    for (int u = 0; u < QB; ++u) {
+      const int e = tid + u * 128;
+      if (TB) {
+        *reinterpret_cast<uint2*>(&Bs[e / (BK / 4)][4 * (e % (BK / 4))]) =
+            make_uint2(pack_bf16(qb[u].x, qb[u].y), pack_bf16(qb[u].z, qb[u].w));
+      } else {
+        const int nn = 4 * (e / BK), kk = e % BK;
+        Bs[nn][kk] = __float2bfloat16_rn(qb[u].x);
+        Bs[nn + 1][kk] = __float2bfloat16_rn(qb[u].y);
+        Bs[nn + 2][kk] = __float2bfloat16_rn(qb[u].z);
+        Bs[nn + 3][kk] = __float2bfloat16_rn(qb[u].w);
+      }
+    }
+  };
+  float ra[VEC ? 1 : PA][2], rb[VEC ? 1 : PB][2];
+  auto loads = [&](int k0) {
 #pragma unroll
     for (int u = 0; u < PA; ++u) {
       const int e = tid + u * 128;
@@ -154,7 +207,7 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs a) {
     }
   };
   // stage A (BM x BK) and B (BN x BK), k contiguous in shared memory
-  auto store = [&]() {
+  auto stores = [&]() {
 #pragma unroll
     for (int u = 0; u < PA; ++u) {
       const int e = tid + u * 128;
@@ -181,9 +234,14 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs a) {
     }
   };
 
+  auto load = [&](int k0) {
+    if constexpr (VEC) loadq(k0);
+    else loads(k0);
+  };
   if (kbeg < kend) load(kbeg);
   for (int k0 = kbeg; k0 < kend; k0 += BK) {
-    store();
+    if constexpr (VEC) storeq();
+    else stores();
     __syncthreads();
     if (k0 + BK < kend) load(k0 + BK);
 #pragma unroll
@@ -239,12 +297,24 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs a) {
       }
 }
 
+// Whether both operands can be read in aligned quads that end where the
+// operand does: K (a quad along k; the split ranges start at multiples of BK)
+// and, for B from [k][n], N multiples of 4, and every row and batch element
+// 16-byte aligned.  Rows of A are M and need no multiple.
+bool gemm_vec(bool ta, bool tb, const GemmArgs& a) {
+  const auto al = [](const float* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; };
+  return !ta && a.K % 4 == 0 && (tb || a.N % 4 == 0) && a.lda % 4 == 0 && a.ldb % 4 == 0 && a.sA % 4 == 0 &&
+         a.sB % 4 == 0 && al(a.A) && al(a.B);
+}
 void gemm(cudaStream_t s, bool ta, bool tb, int batch, const GemmArgs& a) {
   dim3 grid((a.N + BN - 1) / BN, (a.M + BM - 1) / BM, batch * a.splits);
-  if (!ta && !tb) k_gemm<false, false><<<grid, 128, 0, s>>>(a);
-  else if (ta && !tb) k_gemm<true, false><<<grid, 128, 0, s>>>(a);
-  else if (!ta && tb) k_gemm<false, true><<<grid, 128, 0, s>>>(a);
-  else k_gemm<true, true><<<grid, 128, 0, s>>>(a);
+  const bool vec = gemm_vec(ta, tb, a);
+  if (!ta && !tb && vec) k_gemm<false, false, true><<<grid, 128, 0, s>>>(a);
+  else if (!ta && tb && vec) k_gemm<false, true, true><<<grid, 128, 0, s>>>(a);
+  else if (!ta && !tb) k_gemm<false, false, false><<<grid, 128, 0, s>>>(a);
+  else if (ta && !tb) k_gemm<true, false, false><<<grid, 128, 0, s>>>(a);
+  else if (!ta && tb) k_gemm<false, true, false><<<grid, 128, 0, s>>>(a);
+  else k_gemm<true, true, false><<<grid, 128, 0, s>>>(a);
 }
 
 GemmArgs gargs(int M, int N, int K, const float* A, long long lda, long long sA, const float* B, long long ldb,
