@@ -294,9 +294,14 @@ int prepare_film(mm_ctx* c) {
   c->film_spec = nullptr;
   if (!film_plan(c->g, &c->film)) return MM_OK;
   const size_t bytes = 3 * (size_t)c->g.nz * c->g.ny * c->g.hxs * sizeof(float2);
-  MM_CUDA(cudaMalloc((void**)&c->film_spec, bytes));
+  // (without room for its buffers the context steps with the stage kernels)
+  if (cudaMalloc((void**)&c->film_spec, bytes) != cudaSuccess ||
+      (!c->film_sync && cudaMalloc((void**)&c->film_sync, sizeof(FilmSync)) != cudaSuccess)) {
+    (void)cudaGetLastError();
+    c->film = FilmPlan();
+    return MM_OK;
+  }
   MM_CUDA(cudaMemsetAsync(c->film_spec, 0, bytes, c->stream));
-  if (!c->film_sync) MM_CUDA(cudaMalloc((void**)&c->film_sync, sizeof(FilmSync)));
   MM_CUDA(cudaMemsetAsync(c->film_sync, 0, sizeof(FilmSync), c->stream));
   MM_CUDA(cudaStreamSynchronize(c->stream));
   return MM_OK;
