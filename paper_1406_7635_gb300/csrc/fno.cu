@@ -397,6 +397,7 @@ __global__ void k_yexpand(int S, int C, int H, int J, int Mx, const float2* __re
 // kernels above walk a whole column of global memory per thread, which is
 // latency-bound.  Same summation order per output (y, resp. j, ascending).
 constexpr int kYNT = 256;
+constexpr int kYCmax = 64;   // most rows per stage (ysum), per block (yexpand)
 constexpr int kYR = 8;       // most outputs per thread of one column k
 constexpr int kXParts = 4;   // most split-K slices of the x partial DFT products
 constexpr int kYSplit = 8;   // most row ranges of the tiled y product
@@ -410,7 +411,10 @@ constexpr int kYSplit = 8;   // most row ranges of the tiled y product
 // column, jj, jj + JT, ..: one read of x serves them all and the reads of f
 // are the same in most of a warp.  With this and the same in k_yexpand_t a
 // 512 x 512 forward pass of width 32, 24 modes takes 537 us (556 at one output
-// per thread), the gradient of four such samples 4.17 ms (4.40).
+// per thread), the gradient of four such samples 4.17 ms (4.40).  Staging f by
+// asynchronous copies beside the reads of x, without a division per value, took
+// the forward pass from 484 to 462 us (with the 16-byte GEMM loads and the
+// packed layer kernel in place).
 template <int R>
 __global__ void __launch_bounds__(kYNT) k_ysum_t(int H, int J, int Mx, int JB, int YC, int YR,
                                                const float* __restrict__ X, bool x_blocked, int parts,
@@ -428,9 +432,17 @@ __global__ void __launch_bounds__(kYNT) k_ysum_t(int H, int J, int Mx, int JB, i
 #pragma unroll
   for (int r = 0; r < R; ++r) re[r] = im[r] = 0.f;
   const int ybeg = blockIdx.z * YR, yend = min(H, ybeg + YR);
+  const float cs = conj_f ? -1.f : 1.f;
   Y += blockIdx.z * y_stride;
   for (int y0 = ybeg; y0 < yend; y0 += YC) {
     const int yn = min(YC, yend - y0);
+    // f by asynchronous copies beside the reads of x (a row of at most
+    // kYCmax values per kYCmax threads; frequencies past J: zero, not written)
+    for (int a = tid / kYCmax, yy = tid % kYCmax; a < JB; a += kYNT / kYCmax) {
+      if (yy >= yn) break;
+      if (a < jn) cp_async_8(&fs[a * YC + yy], &F[(long long)(j0 + a) * H + y0 + yy]);
+      else fs[a * YC + yy] = make_float2(0.f, 0.f);
+    }
     for (int e = tid; e < yn * Mx; e += kYNT) {
       const int yy = e / Mx, kk = e % Mx;
       const long long ri = sc * H + y0 + yy;
@@ -447,22 +459,18 @@ __global__ void __launch_bounds__(kYNT) k_ysum_t(int H, int J, int Mx, int JB, i
       }
       xs[yy * Mx + kk] = v;
     }
-    for (int e = tid; e < JB * yn; e += kYNT) {   // (frequencies past J: zero, not written)
-      const int a = e / yn, yy = e % yn;
-      float2 f = a < jn ? F[(long long)(j0 + a) * H + y0 + yy] : make_float2(0.f, 0.f);
-      if (conj_f) f.y = -f.y;
-      fs[a * YC + yy] = f;
-    }
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
     __syncthreads();
     if (mine) {
 #pragma unroll 2
       for (int yy = 0; yy < yn; ++yy) {
         const float2 x = xs[yy * Mx + k];
+        const float2 xc = make_float2(cs * x.x, cs * x.y);
 #pragma unroll
         for (int r = 0; r < R; ++r) {
           const float2 f = fs[(jj + JT * r) * YC + yy];
-          re[r] = fmaf(f.x, x.x, fmaf(-f.y, x.y, re[r]));
-          im[r] = fmaf(f.x, x.y, fmaf(f.y, x.x, im[r]));
+          re[r] = fmaf(f.x, x.x, fmaf(-f.y, xc.y, re[r]));
+          im[r] = fmaf(f.x, x.y, fmaf(f.y, xc.x, im[r]));
         }
       }
     }
@@ -501,10 +509,8 @@ __global__ void __launch_bounds__(kYNT) k_yexpand_t(int H, int J, int Mx, int YB
   const int y0 = blockIdx.x * YB, yn = min(YB, H - y0);
   const int tid = threadIdx.x;
   for (int e = tid; e < J * Mx; e += kYNT) cp_async_8(&os[e], &O[sc * J * Mx + e]);
-  for (int e = tid; e < J * yn; e += kYNT) {
-    const int j = e / yn, yy = e % yn;
+  for (int j = tid / kYCmax, yy = tid % kYCmax; j < J && yy < yn; j += kYNT / kYCmax)
     cp_async_8(&fs[j * YB + yy], &F[(long long)j * H + y0 + yy]);
-  }
   asm volatile("cp.async.wait_all;\n" ::: "memory");
   __syncthreads();
   const float cs = conj_f ? -1.f : 1.f;
@@ -521,12 +527,12 @@ __global__ void __launch_bounds__(kYNT) k_yexpand_t(int H, int J, int Mx, int YB
 #pragma unroll 2
     for (int j = 0; j < J; ++j) {
       const float2 o = os[j * Mx + k];
+      const float2 oc = make_float2(cs * o.x, cs * o.y);
 #pragma unroll
       for (int r = 0; r < R; ++r) {
-        float2 f = fs[j * YB + fr[r]];
-        f.y *= cs;
-        re[r] = fmaf(f.x, o.x, fmaf(-f.y, o.y, re[r]));
-        im[r] = fmaf(f.x, o.y, fmaf(f.y, o.x, im[r]));
+        const float2 f = fs[j * YB + fr[r]];
+        re[r] = fmaf(f.x, o.x, fmaf(-f.y, oc.y, re[r]));
+        im[r] = fmaf(f.x, o.y, fmaf(f.y, oc.x, im[r]));
       }
     }
 #pragma unroll
@@ -556,7 +562,7 @@ YTile ytile(int S, int C, int H, int J, int Mx, int sms) {
     const int jt = std::min(J, std::min(64, kYNT / Mx));
     t.R = std::min(kYR, (J + jt - 1) / jt);
     t.JB = jt * t.R;
-    t.YC = std::max(1, std::min(std::min(64, 2048 / Mx), 6144 / (Mx + t.JB)));
+    t.YC = std::max(1, std::min(std::min(kYCmax, 2048 / Mx), 6144 / (Mx + t.JB)));
     // row ranges until about four blocks per multiprocessor, at least a stage each
     const long long blocks = (long long)((J + t.JB - 1) / t.JB) * S * C;
     const long long want = (4LL * sms + blocks - 1) / blocks;
@@ -566,7 +572,7 @@ YTile ytile(int S, int C, int H, int J, int Mx, int sms) {
   t.YB = 0;
   if ((long long)S * C <= 65535 && J * Mx <= 4096) {
     const int yb = (6144 - J * Mx) / J;   // (J Mx + J YB) float2 <= 48 KB
-    t.YB = std::min(H, std::min(64, yb));
+    t.YB = std::min(H, std::min(kYCmax, yb));
     if (t.YB < 1) t.YB = 0;
     const int yt = std::max(1, kYNT / Mx);   // (one pass of the block's threads)
     t.RB = std::max(1, std::min(kYR, (t.YB + yt - 1) / yt));
