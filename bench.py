@@ -600,7 +600,7 @@ def run_ours(args, rank, world, local_rank):
         cf, df, _, _, _ = timed_steps(pf, K, W)
         general["grains_256x256x1_pbc_x"] = {
             "value": pf.ncells * K * world / reduce_max(df), "unit": "cell-steps/s", "ms_per_step": df / K * 1e3,
-            "what": "periodic x (4 images each side): general stage kernels + cyclic x transform"}
+            "what": "periodic x (4 images each side): cyclic x transform, persistent film kernel"}
         cf.close()
         out["general_path"] = general
     if args.batch:
