@@ -128,7 +128,10 @@ int mm_enable_terms(mm_ctx* ctx, int demag, int exch, int anis, int zeeman,
  * the convolution along that axis becomes cyclic (no padding) and the
  * exchange and DMI stencils wrap around.  A periodic axis needs 1 cell or a
  * power of two >= 4 cells (else MM_ERR_ARG).  Rebuilds the demag kernel;
- * keeps m, t, the materials and the geometry mask.  (0, 0, 0) at creation. */
+ * keeps m, t, the materials and the geometry mask.  (0, 0, 0) at creation.
+ * When it fails after the argument checks (MM_ERR_OOM, MM_ERR_CUDA) the
+ * context keeps its state but has no buffers for the grid: calls that step or
+ * evaluate fields return MM_ERR_STATE until a later mm_set_pbc succeeds. */
 int mm_set_pbc(mm_ctx* ctx, int px, int py, int pz);
 
 /* Spin-transfer torques added to dm/dt (off at creation): Zhang-Li,

@@ -86,6 +86,7 @@ struct mm_ctx {
   float2* film_spec = nullptr;
   FilmSync* film_sync = nullptr;
   int method = 0;                // host copy of DevState::method
+  bool usable = true;            // the convolution's buffers are those of the grid (see mm_set_pbc)
   bool lut_dirty = true;
   bool m_set = false;
   bool k1_valid = false;
@@ -123,6 +124,11 @@ int write_state(mm_ctx* c) {
   MM_CUDA(cudaStreamSynchronize(c->stream));
   c->st_fresh = true;
   return MM_OK;
+}
+
+// whether fields can be evaluated; not after a set_pbc that failed
+int check_usable(const mm_ctx* c) {
+  return c->usable ? MM_OK : fail(MM_ERR_STATE, "the last set_pbc failed: the context has no buffers for its grid");
 }
 
 // the host mirror of the device state, read back only if a stepping kernel
@@ -480,7 +486,9 @@ int drive_film(mm_ctx* c, int mode, long long nsteps, double t_end) {
 
 int drive(mm_ctx* c, int mode, long long nsteps, double t_end) {
   if (!c->m_set) return fail(MM_ERR_STATE, "m has not been set");
-  int rc = flush_luts(c);
+  int rc = check_usable(c);
+  if (rc) return rc;
+  rc = flush_luts(c);
   if (rc) return rc;
   if (film_path(c)) return drive_film(c, mode, nsteps, t_end);
   rc = build_graph(c);
@@ -514,7 +522,9 @@ int drive(mm_ctx* c, int mode, long long nsteps, double t_end) {
 }
 
 int eval_field(mm_ctx* c, int mode) {
-  int rc = flush_luts(c);
+  int rc = check_usable(c);
+  if (rc) return rc;
+  rc = flush_luts(c);
   if (rc) return rc;
   rc = read_state(c);
   if (rc) return rc;
@@ -1053,17 +1063,28 @@ int mm_set_pbc(mm_ctx* c, int px, int py, int pz) {
   Geom g = make_geom(c->g.nx, c->g.ny, c->g.nz, c->dx, c->dy, c->dz, pbc);
   if (!fused_plan(g)) large_plan(g);
   MM_CUDA(cudaStreamSynchronize(c->stream));
-  // buffers whose size depends on the transform lengths
+  // Everything whose size or plan depends on the transform lengths goes
+  // first, the film kernel's plan with it: a failure below leaves a context
+  // that refuses to evaluate fields (check_usable), not one that launches the
+  // old plan on the new grid.
+  c->usable = false;
+  c->graph_valid = false;
+  c->k1_valid = false;
   Buffers& b = c->b;
-  void* old[] = {b.spec, b.kt, b.ktf, b.ms2, b.part};
+  void* old[] = {b.spec, b.kt, b.ktf, b.ms2, b.part, c->yzt, c->film_spec};
   for (void* p : old)
     if (p) cudaFree(p);
   b.spec = nullptr;
   b.kt = b.ktf = nullptr;
   b.ms2 = nullptr;
   b.part = nullptr;
-  c->graph_valid = false;
-  c->k1_valid = false;
+  c->yzt = nullptr;
+  c->yz3 = false;
+  c->y2d = false;
+  c->film_spec = nullptr;
+  c->film = FilmPlan();
+  c->maps = RsMaps{};
+  c->g = g;
   const size_t vec = 3 * (size_t)g.n * sizeof(float);
   cudaError_t e = cudaMalloc((void**)&b.spec, 3 * (size_t)g.sc * sizeof(float2));
   if (e == cudaSuccess) e = cudaMemsetAsync(b.spec, 0, 3 * (size_t)g.sc * sizeof(float2), c->stream);
@@ -1076,17 +1097,12 @@ int mm_set_pbc(mm_ctx* c, int px, int py, int pz) {
   if (e == cudaSuccess) e = build_kernel_spectrum(g, c->dx, c->dy, c->dz, b.kt, c->stream);
   if (e == cudaSuccess && g.fused) launch_kt_transpose(g, b.kt, b.ktf, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-  c->g = g;
   if (e == cudaSuccess) {
-    // the (y, z) buffer's size follows the transform lengths
-    if (c->yzt) {
-      cudaFree(c->yzt);
-      c->yzt = nullptr;
-    }
-    c->yz3 = false;
-    c->y2d = false;
     const int rc = apply_yz_choice(c);
-    if (rc) return rc;
+    if (rc) {
+      (void)cudaGetLastError();
+      return rc;
+    }
     // one convolution outside any capture (launch attributes), as at creation
     Buffers nb = b;
     nb.st = nullptr;
@@ -1096,10 +1112,15 @@ int mm_set_pbc(mm_ctx* c, int px, int py, int pz) {
   }
   if (e == cudaSuccess && g.fused && g.pbcx == 0) e = prepare_rowstage(g);
   if (e == cudaSuccess) rowstage_maps(g, b, &c->maps);
-  if (e != cudaSuccess)
+  if (e != cudaSuccess) {
+    (void)cudaGetLastError();
     return fail(e == cudaErrorMemoryAllocation ? MM_ERR_OOM : MM_ERR_CUDA,
                 std::string("set_pbc: ") + cudaGetErrorString(e));
-  return prepare_film(c);
+  }
+  const int rc = prepare_film(c);
+  if (rc) return rc;
+  c->usable = true;
+  return MM_OK;
 }
 
 int mm_get_max_torque(mm_ctx* c, double* tau_max) {
@@ -1350,7 +1371,9 @@ int mm_demag_tensor(int device, double dx, double dy, double dz, int n, const in
 
 int mm_demag_apply(mm_ctx* c, const float* m, float* b) {
   if (!c || !m || !b) return fail(MM_ERR_ARG, "NULL argument");
-  int rc = flush_luts(c);
+  int rc = check_usable(c);
+  if (rc) return rc;
+  rc = flush_luts(c);
   if (rc) return rc;
   Buffers nb = c->b;
   nb.st = nullptr;
@@ -1397,10 +1420,12 @@ int mm_surrogate_train(mm_ctx* c, mm_fno* net, double ms_ref, int n_pairs, int t
   if (!fno_matches(net, c->g)) return fail(MM_ERR_ARG, "surrogate grid differs from the context (2-D, same nx, ny)");
   if (!(ms_ref > 0) || n_pairs < 1 || traj_len < 1 || steps_between < 0 || epochs < 0 || batch < 1 || !(lr > 0))
     return fail(MM_ERR_ARG, "bad training settings");
+  int rc = check_usable(c);
+  if (rc) return rc;
   const long long n3 = 3 * c->g.n;
   // save state
   std::vector<float> m_save(n3);
-  int rc = mm_get_m(c, m_save.data());
+  rc = mm_get_m(c, m_save.data());
   if (rc) return rc;
   double t_save, dt_save;
   rc = mm_get_time(c, &t_save, &dt_save);
@@ -1531,10 +1556,12 @@ int mm_set_yz_kernels(mm_ctx* c, int which, int* active) {
   if (which == 2 && (large_grid(c->g) || (!yz3_plan(c->g) && !y2d_plan(c->g))))
     return fail(MM_ERR_ARG, "the register-resident (y, z) kernels need open y and z axes and, in 3-D, py >= 32 and "
                             "16 <= pz <= 64, in 2-D py of 128, 256 or 512");
+  int rc = check_usable(c);
+  if (rc) return rc;
   MM_CUDA(cudaStreamSynchronize(c->stream));
   c->yz_req = which;
   c->graph_valid = false;   // the captured attempt holds the previous kernels
-  const int rc = apply_yz_choice(c);
+  rc = apply_yz_choice(c);
   if (rc) return rc;
   if (c->yz3 || c->y2d) {
     // one convolution outside any capture (launch attributes)
@@ -1551,8 +1578,10 @@ int mm_set_yz_kernels(mm_ctx* c, int which, int* active) {
 int mm_profile_attempts(mm_ctx* c, int attempts, int max, int* kinds, double* us, int* n_out) {
   if (!c || attempts < 1 || max < 1 || !kinds || !us || !n_out) return fail(MM_ERR_ARG, "bad profiling arguments");
   if (!c->m_set) return fail(MM_ERR_STATE, "m has not been set");
+  int rc = check_usable(c);
+  if (rc) return rc;
   if (!rowstage_path(c)) return fail(MM_ERR_STATE, "profiling covers the fused row-stage path only");
-  int rc = flush_luts(c);
+  rc = flush_luts(c);
   if (rc) return rc;
   // launch positions of one attempt: the prep kernel, then per stage the
   // (y, z) kernel(s) (with demag), the earlier-stage sums (here in line, in

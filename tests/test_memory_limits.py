@@ -1,0 +1,107 @@
+"""What the library does when device memory is short, on the host: its objects
+linked with a CUDA runtime whose device memory is host memory with a settable
+capacity and whose kernels do not run (fake_cudart.cpp)."""
+import ctypes
+import importlib.util
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+PKG = os.path.join(os.path.dirname(HERE), "paper_1406_7635_gb300")
+MM_ERR_OOM, MM_ERR_STATE = -3, -7
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    """The binding over the library with the test's runtime; .rt its controls."""
+    from paper_1406_7635_gb300 import build as b
+    b.build()
+    objs = [os.path.join(b.OUT, u.replace(".cu", ".o")) for u in b.UNITS]
+    if not all(os.path.exists(o) for o in objs):
+        b.build(force=True)
+    lib = str(tmp_path_factory.mktemp("fake") / "libmm_fake.so")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(b._nvcc())), "include")
+    subprocess.run(["g++", "-O1", "-std=c++17", "-fPIC", "-shared", "-Wl,-Bsymbolic", "-I" + cuda, "-o", lib,
+                    os.path.join(HERE, "fake_cudart.cpp"), *objs], check=True)
+    spec = importlib.util.spec_from_file_location("paper_1406_7635_gb300.mm_fake", os.path.join(PKG, "mm.py"))
+    mod = importlib.util.module_from_spec(spec)
+    keep, b.LIB = b.LIB, lib
+    try:
+        spec.loader.exec_module(mod)
+    finally:
+        b.LIB = keep
+    rt = mod._lib
+    rt.fake_set_capacity.argtypes = [ctypes.c_size_t]
+    rt.fake_fail_at.argtypes = [ctypes.c_longlong]
+    rt.fake_used.restype = rt.fake_peak.restype = ctypes.c_size_t
+    rt.fake_launched.restype = ctypes.c_char_p
+    mod.rt = rt
+    return mod
+
+
+@pytest.fixture(autouse=True)
+def unlimited(fake):
+    def free():
+        fake.rt.fake_set_capacity((1 << 64) - 1)
+        fake.rt.fake_fail_at(-1)
+        fake.rt.fake_no_cooperative(0)
+        fake.rt.fake_launched()
+    free()
+    yield
+    free()
+
+
+def kernels(fake):
+    return fake.rt.fake_launched().decode()
+
+
+def context(fake, shape):
+    ctx = fake.Context(*shape, 2e-9, 2e-9, 2e-9)
+    ctx.set_material(0, 8e5, 1.3e-11, 0.1)
+    m = np.zeros((3,) + ctx.shape, np.float32)
+    m[0] = 1.0
+    ctx.set_m(m)
+    return ctx
+
+
+def field_calls(fake, ctx):
+    n = np.zeros((3,) + ctx.shape, np.float32)
+    p = n.ctypes.data_as(ctypes.c_void_p)
+    return [lambda: ctx.step(1), lambda: ctx.run(1e-12), ctx.get_bdemag, ctx.get_beff, ctx.get_torque, ctx.get_energies,
+            ctx.get_max_torque, lambda: ctx.set_yz_kernels(1), lambda: ctx.profile_attempts(1), lambda: ctx.relax(10),
+            lambda: fake._check(fake.mm_demag_apply(ctx.h, p, p))]
+
+
+# a film and a thin stack (persistent kernel), a cluster grid, a large grid
+@pytest.mark.parametrize("shape", [(64, 16, 1), (32, 32, 4), (32, 32, 16), (32, 20, 64)])
+@pytest.mark.parametrize("pbc", [(1, 0, 0), (0, 0, 0)])
+def test_a_failed_set_pbc_leaves_an_error_not_a_stale_plan(fake, shape, pbc):
+    """Whichever of its allocations fails, a context whose set_pbc failed runs
+    no kernel until a later set_pbc succeeds: its buffers and its film plan
+    are not those of its grid."""
+    ctx = context(fake, shape)
+    failed = 0
+    for k in range(40):
+        fake.rt.fake_fail_at(k)
+        try:
+            ctx.set_pbc(*pbc)
+        except fake.MMError as e:
+            assert e.code == MM_ERR_OOM
+            fake.rt.fake_fail_at(-1)
+            kernels(fake)
+            for call in field_calls(fake, ctx):
+                with pytest.raises(fake.MMError) as ei:
+                    call()
+                assert ei.value.code == MM_ERR_STATE
+            assert kernels(fake) == ""
+            ctx.get_m()              # (the state is there)
+            failed += 1
+        fake.rt.fake_fail_at(-1)
+        ctx.set_pbc(*pbc)            # succeeds again
+        ctx.step(1)
+        ctx.get_bdemag()
+    assert failed >= 5               # spectrum, octant and the tensor's work space
+    ctx.close()
