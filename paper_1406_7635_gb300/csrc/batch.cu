@@ -526,6 +526,7 @@ int mm_batch_create(mm_batch** out, int n, const mm_instance_spec* specs, int de
   B->n = n;
   auto cleanup = [&](int code) {
     mm_batch_destroy(B);
+    (void)cudaGetLastError();   // (reported; the caller's next call starts without it)
     return code;
   };
   // group into shape classes

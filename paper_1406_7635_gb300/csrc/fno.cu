@@ -1555,7 +1555,11 @@ int mm_fno_create(mm_fno** out, int H, int W, const mm_fno_cfg* cfg, int device,
   f->bwd_pw = bwd_prepare(C, 2 * Mx);
   f->C = C; f->L = L; f->Mx = Mx; f->My = My; f->H = H; f->W = W; f->J = 2 * My; f->Smax = Smax;
   f->N = (long long)H * W;
-  auto cleanup = [&](int code) { mm_fno_destroy(f); return code; };
+  auto cleanup = [&](int code) {
+    mm_fno_destroy(f);
+    (void)cudaGetLastError();   // (reported; the caller's next call starts without it)
+    return code;
+  };
   // parameter layout
   long long o = 0;
   auto add = [&](long long n) { f->off.push_back(o); o += n; };

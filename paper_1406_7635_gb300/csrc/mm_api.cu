@@ -611,6 +611,7 @@ int mm_create(mm_ctx** out, int nx, int ny, int nz, double dx, double dy, double
 
   auto cleanup = [&](int code) {
     mm_destroy(c);
+    (void)cudaGetLastError();   // (reported; the caller's next call starts without it)
     return code;
   };
   cudaError_t e = cudaSuccess;

@@ -105,3 +105,35 @@ def test_a_failed_set_pbc_leaves_an_error_not_a_stale_plan(fake, shape, pbc):
         ctx.get_bdemag()
     assert failed >= 5               # spectrum, octant and the tensor's work space
     ctx.close()
+
+
+def make(fake, kind):
+    """The allocations of one creation, which is closed again."""
+    if kind == "context":
+        obj = fake.Context(40, 40, 9, 2e-9, 2e-9, 2e-9)
+    elif kind == "film":
+        obj = fake.Context(64, 40, 1, 2e-9, 2e-9, 2e-9)
+    elif kind == "batch":
+        obj = fake.Batch([dict(nx=32, ny=16, nz=nz, dx=2e-9, dy=2e-9, dz=2e-9, msat=8e5, aex=1e-11, alpha=0.1,
+                               bext=(0, 0, 0)) for nz in (1, 2)])
+    else:
+        obj = fake.FNO(32, 32, width=32, layers=2, modes_x=8, modes_y=8, max_batch=2)
+    obj.close()
+
+
+@pytest.mark.parametrize("kind", ["context", "film", "batch", "network"])
+def test_a_failed_creation_keeps_nothing(fake, kind):
+    """MM_ERR_OOM at creation gives everything back, its error included: the
+    next creation in the same thread succeeds."""
+    base, failed = fake.rt.fake_used(), 0
+    for k in range(80):
+        fake.rt.fake_fail_at(k)
+        try:
+            make(fake, kind)
+        except fake.MMError as e:
+            assert e.code == MM_ERR_OOM
+            failed += 1
+        assert fake.rt.fake_used() == base
+        fake.rt.fake_fail_at(-1)
+        make(fake, kind)
+    assert failed > 10
