@@ -269,6 +269,37 @@ int apply_yz_choice(mm_ctx* c) {
   return MM_OK;
 }
 
+// Moves a grid beyond the cluster kernel's planes to the three kernels and
+// the row-stage kernels (large_plan) if there is room for what they need
+// beside the general convolution's buffers: those are in place, the work space
+// of the kernel spectrum has been given back, so a grid that the general
+// convolution has room for is served by it at least.  256 x 256 x 64 cells
+// take 0.4 GB more, 512 x 512 x 64 cells 1.6 GB.
+void prepare_large(mm_ctx* c) {
+  Geom g = c->g;
+  if (!large_plan(g)) return;
+  Buffers& b = c->b;
+  const size_t vec = 3 * (size_t)g.n * sizeof(float), oct = 6 * (size_t)g.hkx * g.hky * g.hkz * sizeof(float);
+  cudaError_t e = cudaMalloc((void**)&c->yzt, yz3_bytes(g));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&b.ktf, oct);
+  if (e == cudaSuccess) e = cudaMalloc((void**)&b.ms2, vec);
+  if (e == cudaSuccess) e = cudaMalloc((void**)&b.part, vec);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b.ms2, 0, vec, c->stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(b.part, 0, vec, c->stream);
+  if (e != cudaSuccess) {
+    (void)cudaGetLastError();
+    cudaFree(c->yzt);
+    cudaFree(b.ktf);
+    cudaFree(b.ms2);
+    cudaFree(b.part);
+    c->yzt = nullptr;
+    b.ktf = b.ms2 = b.part = nullptr;
+    return;
+  }
+  c->g = g;
+  launch_kt_transpose(g, b.kt, b.ktf, c->stream);
+}
+
 // demag field of the stage input: exact convolution, or the surrogate
 void enqueue_demag(mm_ctx* c) {
   if (!c->T.demag) return;
@@ -599,7 +630,7 @@ int mm_create(mm_ctx** out, int nx, int ny, int nz, double dx, double dy, double
   c->dz = dz;
   c->g = make_geom(nx, ny, nz, dx, dy, dz);
   Geom& g = c->g;
-  if (!fused_plan(g)) large_plan(g);
+  fused_plan(g);
   for (int r = 0; r < kRegions; ++r) {
     std::memset(&c->mat[r], 0, sizeof(mm_material));
     c->mat[r].gamma_ll = kGamma;
@@ -675,6 +706,7 @@ int mm_create(mm_ctx** out, int nx, int ny, int nz, double dx, double dy, double
   if (e != cudaSuccess)
     return cleanup(fail(e == cudaErrorMemoryAllocation ? MM_ERR_OOM : MM_ERR_CUDA,
                         std::string("kernel precompute: ") + cudaGetErrorString(e)));
+  prepare_large(c);
   // device state defaults (Sec. IV: MaxErr 1e-5, headroom 0.8)
   DevState& s = *c->st_host;
   std::memset(&s, 0, sizeof(DevState));
@@ -1062,7 +1094,7 @@ int mm_set_pbc(mm_ctx* c, int px, int py, int pz) {
       return fail(MM_ERR_ARG, "a periodic axis needs 1 cell or a power of two >= 4 cells");
   }
   Geom g = make_geom(c->g.nx, c->g.ny, c->g.nz, c->dx, c->dy, c->dz, pbc);
-  if (!fused_plan(g)) large_plan(g);
+  fused_plan(g);
   MM_CUDA(cudaStreamSynchronize(c->stream));
   // Everything whose size or plan depends on the transform lengths goes
   // first, the film kernel's plan with it: a failure below leaves a context
@@ -1099,6 +1131,7 @@ int mm_set_pbc(mm_ctx* c, int px, int py, int pz) {
   if (e == cudaSuccess && g.fused) launch_kt_transpose(g, b.kt, b.ktf, c->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e == cudaSuccess) {
+    prepare_large(c);
     const int rc = apply_yz_choice(c);
     if (rc) {
       (void)cudaGetLastError();
@@ -1111,8 +1144,8 @@ int mm_set_pbc(mm_ctx* c, int px, int py, int pz) {
     e = cudaStreamSynchronize(c->stream);
     if (e == cudaSuccess) e = cudaGetLastError();
   }
-  if (e == cudaSuccess && g.fused && g.pbcx == 0) e = prepare_rowstage(g);
-  if (e == cudaSuccess) rowstage_maps(g, b, &c->maps);
+  if (e == cudaSuccess && c->g.fused && g.pbcx == 0) e = prepare_rowstage(c->g);
+  if (e == cudaSuccess) rowstage_maps(c->g, b, &c->maps);
   if (e != cudaSuccess) {
     (void)cudaGetLastError();
     return fail(e == cudaErrorMemoryAllocation ? MM_ERR_OOM : MM_ERR_CUDA,

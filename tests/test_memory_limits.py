@@ -137,3 +137,69 @@ def test_a_failed_creation_keeps_nothing(fake, kind):
         fake.rt.fake_fail_at(-1)
         make(fake, kind)
     assert failed > 10
+
+
+# kernels of a large grid (the three (y, z) kernels, the row-stage kernels)
+FAST = ("k_zk", "k_rs_")
+
+
+@pytest.mark.parametrize("nx,ny,nz", [(20, 18, 64), (17, 21, 33)])
+def test_a_large_grid_without_room_for_its_kernels_takes_the_general_ones(fake, nx, ny, nz):
+    """At creation and in set_pbc: a failure of any allocation that the
+    general convolution does without leaves a working context, all of them
+    given back; a failure of any other is MM_ERR_OOM, nothing kept."""
+    base = fake.rt.fake_used()
+    ctx = context(fake, (nx, ny, nz))
+    full = fake.rt.fake_used() - base
+    kernels(fake)
+    ctx.step(1)
+    ctx.get_bdemag()
+    names = kernels(fake)
+    assert all(f in names for f in FAST)
+    ctx.close()
+    assert fake.rt.fake_used() == base
+    up = lambda n: 1 << (2 * n - 2).bit_length()  # noqa: E731
+    hx, hy, hz = up(nx) // 2 + 1, up(ny) // 2 + 1, up(nz) // 2 + 1
+    extra = [8 * 3 * hx * nz * up(ny), 24 * hx * hy * hz, 12 * nx * ny * nz, 12 * nx * ny * nz]
+    general = 0
+    for k in range(60):
+        fake.rt.fake_fail_at(k)
+        try:
+            ctx = context(fake, (nx, ny, nz))
+        except fake.MMError as e:
+            assert e.code == MM_ERR_OOM and fake.rt.fake_used() == base
+            continue
+        used = fake.rt.fake_used() - base
+        if used != full:
+            general += 1
+            assert used == full - sum(extra)
+            for _ in range(2):
+                kernels(fake)
+                ctx.step(1)
+                ctx.get_bdemag()
+                names = kernels(fake)
+                assert not any(f in names for f in FAST) and "k_fx" in names
+                assert ctx.set_yz_kernels(0) == 0 and ctx.set_yz_kernels(1) == 0
+            fake.rt.fake_fail_at(-1)
+            ctx.set_pbc(0, 0, 0)     # room again: the fast kernels
+            assert fake.rt.fake_used() - base == full
+            ctx.step(1)
+            names = kernels(fake)
+            assert all(f in names for f in FAST)
+        ctx.close()
+    assert general == len(extra)
+    # set_pbc
+    ctx = context(fake, (nx, ny, nz))
+    general = 0
+    for k in range(20):
+        fake.rt.fake_fail_at(k)
+        try:
+            ctx.set_pbc(0, 0, 0)
+        except fake.MMError:
+            continue
+        if fake.rt.fake_used() - base != full:
+            general += 1
+            assert fake.rt.fake_used() - base == full - sum(extra)
+            ctx.step(1)
+    assert general == len(extra)
+    ctx.close()
