@@ -349,6 +349,11 @@ int prepare_film(mm_ctx* c) {
 // particular ones steps with them, in the stage kernels' graph).
 bool film_path(const mm_ctx* c) { return c->film.rows > 0 && c->T.demag && !c->sur_active && c->yz_req == 0; }
 
+// The film plan counts the whole device's multiprocessors; a stream on a part
+// of them (a green context, a limited MPS client) may refuse the launch.  The
+// context then steps with the stage kernels, as one without a plan.
+constexpr int kFilmRefused = 1;
+
 // one launch of the film kernel: the first stage alone (k1), or up to
 // `attempts` attempts; begin starts a call of `mode`
 int enqueue_film(mm_ctx* c, bool begin, int mode, long long nsteps, double t_end, bool k1, int attempts) {
@@ -384,8 +389,13 @@ int enqueue_film(mm_ctx* c, bool begin, int mode, long long nsteps, double t_end
   // been under it, so a film keeps its behaviour at a given limit)
   a.state_limit = rowstage_path(c) && (c->maps.ok_spec || c->maps.ok_sten);
   a.oct_sm = c->film.oct_sm;
+  const cudaError_t e = launch_film(c->film, a, c->stream);
+  if (e == cudaErrorCooperativeLaunchTooLarge) {
+    (void)cudaGetLastError();
+    return kFilmRefused;
+  }
+  MM_CUDA(e);
   c->launches += 1;
-  MM_CUDA(launch_film(c->film, a, c->stream));
   return MM_OK;
 }
 
@@ -505,6 +515,7 @@ int drive_film(mm_ctx* c, int mode, long long nsteps, double t_end) {
   if (!k1_was_valid) rc = enqueue_film(c, true, mode, nsteps, t_end, true, 1);
   for (int guard = 0; guard < 1000000 && !rc; ++guard) {
     rc = enqueue_film(c, guard == 0 && k1_was_valid, mode, nsteps, t_end, false, kFilmAttempts);
+    if (rc == kFilmRefused && guard > 0) rc = fail(MM_ERR_CUDA, "the film kernel's launch was refused during a call");
     if (rc) break;
     rc = read_state(c);
     if (rc) break;
@@ -521,7 +532,11 @@ int drive(mm_ctx* c, int mode, long long nsteps, double t_end) {
   if (rc) return rc;
   rc = flush_luts(c);
   if (rc) return rc;
-  if (film_path(c)) return drive_film(c, mode, nsteps, t_end);
+  if (film_path(c)) {
+    rc = drive_film(c, mode, nsteps, t_end);
+    if (rc != kFilmRefused) return rc;
+    c->film = FilmPlan();   // (begun anew below: nothing has been stepped)
+  }
   rc = build_graph(c);
   if (rc) return rc;
   c->st_fresh = false;   // the stepping kernels write the device state

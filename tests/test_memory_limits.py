@@ -203,3 +203,21 @@ def test_a_large_grid_without_room_for_its_kernels_takes_the_general_ones(fake, 
             ctx.step(1)
     assert general == len(extra)
     ctx.close()
+
+
+@pytest.mark.parametrize("shape", [(64, 16, 1), (32, 32, 4)])
+def test_a_refused_cooperative_launch_steps_with_the_stage_kernels(fake, shape):
+    """A stream on fewer multiprocessors than the film kernel's blocks need (a
+    partition of the device) refuses its launch: the call runs on the stage
+    kernels' graph, which needs no co-residency, and so do later ones."""
+    ctx = context(fake, shape)
+    kernels(fake)
+    ctx.step(1)
+    assert "k_film" in kernels(fake)
+    fake.rt.fake_no_cooperative(1)
+    for call in (lambda: ctx.step(1), lambda: ctx.run(1e-12)):
+        call()
+        names = kernels(fake)
+        assert "graph" in names and "k_film" not in names
+    ctx.get_bdemag()             # (the refusal is no error of a later call)
+    ctx.close()
