@@ -170,16 +170,19 @@ __host__ __device__ constexpr bool takes(int s, int j) { return j < s && !(s == 
 
 // Effective field (demag + exchange + static Zeeman) and LL torque of stage
 // S, k_S, and what follows from a cell's own slopes while they are at hand:
-// S = 1 .. 5 the cell's input of stage S + 1 (to ms_next; ms is still read by
-// the neighbours), S = 6 its error and new m and the instance's step decision.
+// S = 1 .. 5 the cell's input of stage S + 1, in the place of its field in
+// `fn` (only this thread reads that; ms is still read by the neighbours),
+// S = 6 its error and new m and the instance's step decision.
 // Bound by memory and by the drain between dependent launches: as kernels of
 // their own the next input and the error read k_S and m again and cost six
 // more launches per attempt.  64 instances of 901120 cells in all: 23.92 ms
-// for one picosecond with the states set and read (24.42 ms with them apart).
+// for one picosecond with the states set and read (24.42 ms with them apart);
+// with the next input in the field's place, not a buffer of its own, 23.05 ms
+// (23.31 ms on the same card) and one vector per instance less.
 template <int S>
-__global__ void k_b_stage(Geom g, BPtrs p, const float* __restrict__ ms, float* __restrict__ ms_next,
-                          const float* __restrict__ bd, const InstParams* __restrict__ prm,
-                          InstState* __restrict__ st, double* __restrict__ hist) {
+__global__ void k_b_stage(Geom g, BPtrs p, const float* __restrict__ ms, float* __restrict__ fn,
+                          const InstParams* __restrict__ prm, InstState* __restrict__ st,
+                          double* __restrict__ hist) {
   const int inst = blockIdx.y;
   InstState& I = st[inst];
   if (I.done) return;   // uniform over the instance's blocks
@@ -189,7 +192,7 @@ __global__ void k_b_stage(Geom g, BPtrs p, const float* __restrict__ ms, float* 
   float e = 0.0f;
   if (i < n) {
     const float* __restrict__ m = ms + o;
-    const float* __restrict__ bdo = bd + o;
+    float* __restrict__ fo = fn + o;
     const InstParams P = prm[inst];
     // the cell's m and slopes, loaded together
     float m0[3] = {0.f, 0.f, 0.f}, ks[6][3];
@@ -209,7 +212,7 @@ __global__ void k_b_stage(Geom g, BPtrs p, const float* __restrict__ ms, float* 
     }
     const int x = i % g.nx, y = (i / g.nx) % g.ny, z = i / (g.nx * g.ny);
     const float mx = m[i], my = m[n + i], mz = m[2 * n + i];
-    float bx = bdo[i] + P.b[0], by = bdo[n + i] + P.b[1], bz = bdo[2 * n + i] + P.b[2];
+    float bx = fo[i] + P.b[0], by = fo[n + i] + P.b[1], bz = fo[2 * n + i] + P.b[2];
     auto nb = [&](int j, float id2) {
       const float c = P.exch * id2;
       bx += c * (m[j] - mx);
@@ -230,7 +233,6 @@ __global__ void k_b_stage(Geom g, BPtrs p, const float* __restrict__ ms, float* 
 #pragma unroll
     for (int c = 0; c < 3; ++c) k[c * n + i] = kk[c];
     if constexpr (S >= 1 && S <= 5) {
-      float* __restrict__ out = ms_next + o;
 #pragma unroll
       for (int j = 0; j <= S; ++j) {
         if (!takes(S + 1, j)) continue;
@@ -240,7 +242,7 @@ __global__ void k_b_stage(Geom g, BPtrs p, const float* __restrict__ ms, float* 
         for (int c = 0; c < 3; ++c) m0[c] = fmaf(a, j < S ? ks[j][c] : kk[c], m0[c]);
       }
 #pragma unroll
-      for (int c = 0; c < 3; ++c) out[c * n + i] = m0[c];
+      for (int c = 0; c < 3; ++c) fo[c * n + i] = m0[c];
     }
     if constexpr (S == 6) {
       float ev[3] = {0.f, 0.f, 0.f};
@@ -320,7 +322,6 @@ struct BClass {
   int first = 0;            // offset of its first instance in the state array
   std::vector<int> ids;     // global instance indices
   Buffers b{};
-  float* ms2 = nullptr;     // the other stage input (a stage writes the next one)
   float* msat = nullptr;
   InstParams* prm = nullptr;
   double* hist = nullptr;
@@ -376,28 +377,33 @@ BatchArgs bargs(const mm_batch* B, const BClass& c) {
   return BatchArgs{c.B, c.msat, &B->st[c.first].done, (int)(sizeof(InstState) / sizeof(int))};
 }
 
-// stage S of every unfinished instance of class c from its input in ms[S & 1]
+// The stage inputs: odd stages take theirs from bd, even ones from ms, and
+// the field of a stage goes to the other buffer, which its k_b_stage turns into
+// the next stage's input.
+float* stage_buf(const BClass& c, int s) { return (s & 1) ? c.b.bd : c.b.ms; }
+
+// stage S of every unfinished instance of class c from its input
 template <int S>
 void enqueue_eval(mm_batch* B, BClass& c, cudaStream_t st) {
   const Geom& g = c.g;
   const dim3 grid((unsigned)((g.n + kT - 1) / kT), c.B);
-  float* ms[2] = {c.b.ms, c.ms2};
   Buffers bb = c.b;
   bb.st = nullptr;
-  launch_demag_fused_batch(g, bb, ms[S & 1], st, bargs(B, c));
-  k_b_stage<S><<<grid, kT, 0, st>>>(g, bptrs(c), ms[S & 1], ms[(S + 1) & 1], c.b.bd, c.prm, B->st + c.first, c.hist);
+  bb.bd = stage_buf(c, S + 1);
+  launch_demag_fused_batch(g, bb, stage_buf(c, S), st, bargs(B, c));
+  k_b_stage<S><<<grid, kT, 0, st>>>(g, bptrs(c), stage_buf(c, S), bb.bd, c.prm, B->st + c.first, c.hist);
 }
 
 // k_0 of every unfinished instance of class c at its m
 void enqueue_k1(mm_batch* B, BClass& c, cudaStream_t st) {
   const dim3 grid((unsigned)((c.g.n + kT - 1) / kT), c.B);
-  k_b_stage_input<<<grid, kT, 0, st>>>(c.g, bptrs(c), c.b.ms, B->st + c.first, 0);
+  k_b_stage_input<<<grid, kT, 0, st>>>(c.g, bptrs(c), stage_buf(c, 0), B->st + c.first, 0);
   enqueue_eval<0>(B, c, st);
 }
 
 void enqueue_attempt(mm_batch* B, BClass& c, cudaStream_t st) {
   const dim3 grid((unsigned)((c.g.n + kT - 1) / kT), c.B);
-  k_b_stage_input<<<grid, kT, 0, st>>>(c.g, bptrs(c), c.ms2, B->st + c.first, 1);
+  k_b_stage_input<<<grid, kT, 0, st>>>(c.g, bptrs(c), stage_buf(c, 1), B->st + c.first, 1);
   enqueue_eval<1>(B, c, st);
   enqueue_eval<2>(B, c, st);
   enqueue_eval<3>(B, c, st);
@@ -591,7 +597,6 @@ int mm_batch_create(mm_batch** out, int n, const mm_instance_spec* specs, int de
     alloc((void**)&C.b.m[1], vec);
     for (int j = 0; j < 7; ++j) alloc((void**)&C.b.k[j], vec);
     alloc((void**)&C.b.ms, vec);
-    alloc((void**)&C.ms2, vec);
     alloc((void**)&C.b.bd, vec);
     alloc((void**)&C.b.spec, (size_t)C.B * 3 * g.hx * g.nz * g.ny * sizeof(float2));
     alloc((void**)&C.b.kt, 6 * (size_t)g.hkx * g.hky * g.hkz * sizeof(float));
@@ -657,7 +662,7 @@ int mm_batch_destroy(mm_batch* B) {
   if (B->exec) cudaGraphExecDestroy(B->exec);
   for (BClass& C : B->cls) {
     void* ptrs[] = {C.b.m[0], C.b.m[1], C.b.k[0], C.b.k[1], C.b.k[2], C.b.k[3], C.b.k[4], C.b.k[5], C.b.k[6],
-                    C.b.ms,   C.ms2,    C.b.bd,   C.b.spec, C.b.kt,   C.b.ktf,  C.msat,   C.prm,    C.hist};
+                    C.b.ms,   C.b.bd,   C.b.spec, C.b.kt,   C.b.ktf,  C.msat,   C.prm,    C.hist};
     for (void* p : ptrs)
       if (p) cudaFree(p);
   }

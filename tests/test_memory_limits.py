@@ -221,3 +221,19 @@ def test_a_refused_cooperative_launch_steps_with_the_stage_kernels(fake, shape):
         assert "graph" in names and "k_film" not in names
     ctx.get_bdemag()             # (the refusal is no error of a later call)
     ctx.close()
+
+
+def test_a_batch_holds_eleven_vectors_per_instance(fake):
+    """m twice, seven slopes, and two buffers that are in turn the input and
+    the field of a stage, beside the spectrum."""
+    def held(n):
+        base = fake.rt.fake_used()
+        b = fake.Batch([dict(nx=96, ny=96, nz=4, dx=2e-9, dy=2e-9, dz=2e-9, msat=8e5, aex=1e-11, alpha=0.1,
+                             bext=(0, 0, 0))] * n)
+        used = fake.rt.fake_used() - base
+        b.close()
+        return used
+
+    vec, spec, small = 12 * 96 * 96 * 4, 8 * 3 * 129 * 4 * 96, 1 << 16
+    history = 8 * 4096
+    assert 11 * vec + spec <= held(3) - held(2) <= 11 * vec + spec + history + small
