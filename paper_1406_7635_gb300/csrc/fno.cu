@@ -1608,8 +1608,13 @@ int mm_fno_create(mm_fno** out, int H, int W, const mm_fno_cfg* cfg, int device,
   alloc((void**)&f->dV, (size_t)Smax * C * f->J * Mx * sizeof(float2));
   alloc((void**)&f->Yp, (size_t)kYSplit * Smax * C * f->J * Mx * sizeof(float2));
   alloc((void**)&f->acc, 4 * sizeof(double));
-  if (f->bwd_pw) alloc((void**)&f->part, bwd_part_floats(f) * sizeof(float));
   if (e != cudaSuccess) return cleanup(ffail(e == cudaErrorMemoryAllocation ? MM_ERR_OOM : MM_ERR_CUDA, cudaGetErrorString(e)));
+  // (without room for its partial sums the separate products serve)
+  if (f->bwd_pw && cudaMalloc((void**)&f->part, bwd_part_floats(f) * sizeof(float)) != cudaSuccess) {
+    (void)cudaGetLastError();
+    f->part = nullptr;
+    f->bwd_pw = false;
+  }
   // partial DFT matrices (float64 on the host, rounded once)
   const double pi = 3.14159265358979323846;
   std::vector<float> Fb((size_t)W * 2 * Mx), Gb((size_t)2 * Mx * W);

@@ -237,3 +237,28 @@ def test_a_batch_holds_eleven_vectors_per_instance(fake):
     vec, spec, small = 12 * 96 * 96 * 4, 8 * 3 * 129 * 4 * 96, 1 << 16
     history = 8 * 4096
     assert 11 * vec + spec <= held(3) - held(2) <= 11 * vec + spec + history + small
+
+
+def test_a_network_without_room_for_partial_sums_keeps_the_separate_products(fake):
+    """The fused backward pass needs a buffer that the separate products do
+    without: no room for it is no reason to refuse the network."""
+    u = np.zeros((2, 3, 32, 32), np.float32)
+    p = u.ctypes.data_as(ctypes.c_void_p)
+    created, fused = 0, []
+    for k in range(60):
+        fake.rt.fake_fail_at(k)
+        try:
+            net = fake.FNO(32, 32, width=32, layers=2, modes_x=8, modes_y=8, max_batch=2)
+        except fake.MMError as e:
+            assert e.code == MM_ERR_OOM
+            continue
+        fake.rt.fake_fail_at(-1)
+        kernels(fake)
+        g = np.zeros(net.nparams(), np.float32)
+        loss = ctypes.c_double()
+        for _ in range(2):
+            fake._check(fake.mm_fno_grad(net.h, p, p, 2, g.ctypes.data_as(ctypes.c_void_p), ctypes.byref(loss)))
+        fused.append("k_bwd_pw" in kernels(fake))
+        net.close()
+        created += 1
+    assert created > 10 and fused.count(False) == 1 and not fused[0]
