@@ -956,10 +956,15 @@ int mm_set_fixed_dt_sequence(mm_ctx* c, const double* dts, int n) {
   for (int i = 0; i < n; ++i)
     if (!(dts[i] > 0) || !std::isfinite(dts[i])) return fail(MM_ERR_ARG, "step sizes must be finite and > 0");
   if (n > c->fixed_cap) {
+    // (the sequence in place stays if there is no room: later steps replay it)
+    double* longer = nullptr;
+    const cudaError_t e = cudaMalloc((void**)&longer, (size_t)n * sizeof(double));
+    if (e != cudaSuccess) {
+      (void)cudaGetLastError();
+      return fail(e == cudaErrorMemoryAllocation ? MM_ERR_OOM : MM_ERR_CUDA, "no room for the step sequence");
+    }
     if (c->b.fixed) cudaFree(c->b.fixed);
-    c->b.fixed = nullptr;
-    c->fixed_cap = 0;
-    MM_CUDA(cudaMalloc((void**)&c->b.fixed, (size_t)n * sizeof(double)));
+    c->b.fixed = longer;
     c->fixed_cap = n;
     c->graph_valid = false;   // the error kernel's pointer changed
   }

@@ -262,3 +262,21 @@ def test_a_network_without_room_for_partial_sums_keeps_the_separate_products(fak
         net.close()
         created += 1
     assert created > 10 and fused.count(False) == 1 and not fused[0]
+
+
+def test_a_longer_replay_sequence_without_room_keeps_the_one_there(fake):
+    base = fake.rt.fake_used()
+    ctx = context(fake, (20, 20, 5))
+    ctx.set_fixed_dt_sequence([1e-14] * 4)
+    held = fake.rt.fake_used()
+    fake.rt.fake_fail_at(0)
+    with pytest.raises(fake.MMError) as ei:
+        ctx.set_fixed_dt_sequence([1e-14] * 1000)
+    assert ei.value.code == MM_ERR_OOM
+    assert fake.rt.fake_used() == held      # (steps still replay from the buffer that is there)
+    ctx.step(1)
+    ctx.get_bdemag()                        # (no error left for a later call)
+    ctx.set_fixed_dt_sequence([1e-14] * 1000)
+    assert fake.rt.fake_used() == held + 8 * 996
+    ctx.close()
+    assert fake.rt.fake_used() == base
