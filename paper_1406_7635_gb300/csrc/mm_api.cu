@@ -489,12 +489,14 @@ int build_graph(mm_ctx* c) {
   return MM_OK;
 }
 
-int status_to_code(int status) {
+// film: the status is the film kernel's
+int status_to_code(int status, bool film = false) {
   if (status == MM_ERR_NONFINITE) return fail(MM_ERR_NONFINITE, "non-finite step error (NaN/Inf in m or torque)");
   if (status == MM_ERR_DT_UNDERFLOW) return fail(MM_ERR_DT_UNDERFLOW, "time step fell below dt_min");
   if (status == MM_ERR_TIMEOUT)
-    return fail(MM_ERR_TIMEOUT, "a kernel's bounded wait on its tensor copies expired (the attempt was abandoned; m, t "
-                                "and dt are those before it)");
+    return fail(MM_ERR_TIMEOUT, std::string("a kernel's bounded wait on ") +
+                                    (film ? "the other blocks at a grid barrier" : "its tensor copies") +
+                                    " expired (the attempt was abandoned; m, t and dt are those before it)");
   if (status != 0) return fail(status, "device status error");
   return MM_OK;
 }
@@ -521,7 +523,7 @@ int drive_film(mm_ctx* c, int mode, long long nsteps, double t_end) {
     if (rc) break;
     const DevState& s = *c->st_host;
     c->k1_valid = k1_was_valid || s.call_attempts > 0;
-    if (s.done) return status_to_code(s.status);
+    if (s.done) return status_to_code(s.status, true);
   }
   return rc ? rc : fail(MM_ERR_STATE, "stepping loop did not finish");
 }
