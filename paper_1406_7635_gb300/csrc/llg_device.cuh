@@ -326,55 +326,79 @@ __device__ void check_done(DevState* st) {
 // whose error estimate is of order 2), bounded by dt_max, and
 // at least dt_min after an accepted step; a rejection that would need a step
 // below dt_min ends the call with MM_ERR_DT_UNDERFLOW.
-// (hist null: the accepted step size is not recorded)
-__device__ void controller_core(DevState* st, double* __restrict__ hist) {
-  const double eps = (double)__uint_as_float(st->err_bits);
-  st->err_bits = 0;
-  st->ticket = 0;
+//
+// Its decision stands here once, for the stage kernels (controller_on) and the
+// film kernel.  The growth factor in float32: it only scales dt and is clamped
+// to [0.2, 5].  A float64 pow runs on the GPU's FP64 pipe, slow on this part,
+// in one thread at the end of every attempt: measured on the 128 x 128 x 32
+// step, the last row kernel took 35.6 us with it and 31.1 us without.
+struct StepDecision {
+  double t, dt;
+  int accept, status, done, fixed_idx;
+};
+__device__ __forceinline__ StepDecision step_decide(const DevState& s, float eps) {
+  StepDecision d{s.t, s.dt, 0, 0, 0, s.fixed_idx};
+  if (!(eps <= FLT_MAX)) {
+    d.status = -4;   // MM_ERR_NONFINITE
+    d.done = 1;
+    return d;
+  }
+  const double h = s.h;
+  const bool replay = s.mode == 2;
+  d.accept = replay || eps <= __double2float_rd(s.max_err);   // (eps <= max_err for a float eps)
+  const float ex = s.method == 1 ? 1.0f / 3.0f : 0.2f;
+  const float ratio = (float)s.max_err / eps;   // (inf for a tiny eps)
+  const double factor = eps == 0.0f ? 5.0 : (double)fminf(5.0f, fmaxf(0.2f, (float)s.headroom * powf(ratio, ex)));
+  const double ndt = fmin(h * factor, s.dt_max);
+  if (d.accept) {
+    d.t = s.t + h;
+    if (s.mode == 1 && d.t + 1e-6 * h >= s.t_end) d.t = s.t_end;
+    if (replay) ++d.fixed_idx;
+    else d.dt = fmax(ndt, s.dt_min);
+    if (s.mode == 0) d.done = s.accepted + 1 >= s.target;
+    else if (s.mode == 1) d.done = d.t >= s.t_end;
+    else d.done = d.fixed_idx >= s.fixed_n || s.accepted + 1 >= s.target;
+  } else if (ndt < s.dt_min) {
+    d.status = -5;   // MM_ERR_DT_UNDERFLOW
+    d.done = 1;
+  } else {
+    d.dt = ndt;
+  }
+  return d;
+}
+// the decided attempt's end in the state (status and done stay as an expired
+// wait has set them); the accepted step size goes to hist (null: another block
+// records it)
+__device__ __forceinline__ void step_apply(DevState* st, const StepDecision& d, float eps, double* __restrict__ hist) {
+  if (d.accept && hist && st->hist_n < kHistCap) hist[st->hist_n] = st->h;
   st->evals += st->method == 1 ? 3 : 6;
   st->call_attempts++;
-  st->last_err = eps;
-  if (!(eps <= DBL_MAX)) {
-    st->status = -4;   // MM_ERR_NONFINITE
-    st->done = 1;
-    return;
-  }
-  const double h = st->h;
-  const bool replay = st->mode == 2;
-  const bool accept = replay || eps <= st->max_err;
-  // The growth factor in float32: it only scales dt and is clamped to
-  // [0.2, 5].  A float64 pow runs on the GPU's FP64 pipe, slow on this part,
-  // in one thread at the end of every attempt: measured on the 128 x 128 x 32
-  // step, the last row kernel took 35.6 us with it and 31.1 us without.
-  const float ex = st->method == 1 ? 1.0f / 3.0f : 0.2f;
-  const float ratio = (float)st->max_err / (float)eps;   // eps > 0 below; inf for a tiny eps
-  const double factor = eps == 0.0 ? 5.0 : (double)fminf(5.0f, fmaxf(0.2f, (float)st->headroom * powf(ratio, ex)));
-  const double ndt = fmin(h * factor, st->dt_max);
-  if (accept) {
-    st->t += h;
-    if (st->mode == 1 && st->t + 1e-6 * h >= st->t_end) st->t = st->t_end;
-    st->parity ^= 1;
-    if (hist && st->hist_n < kHistCap) hist[st->hist_n] = h;
-    st->hist_n++;
-    st->accepted++;
-    if (replay) st->fixed_idx++;
-    else st->dt = fmax(ndt, st->dt_min);
-    check_done(st);
-  } else {
-    st->rejected++;
-    if (ndt < st->dt_min) {
-      st->status = -5;   // MM_ERR_DT_UNDERFLOW
-      st->done = 1;
-      return;
+  st->last_err = (double)eps;
+  if (d.status == 0) {
+    if (d.accept) {
+      st->t = d.t;
+      st->parity ^= 1;
+      st->hist_n++;
+      st->accepted++;
+      st->fixed_idx = d.fixed_idx;
+    } else {
+      st->rejected++;
     }
-    st->dt = ndt;
+    st->dt = d.dt;
+  } else {
+    st->status = d.status;
+    if (d.status == -5) st->rejected++;
   }
+  if (d.done) st->done = 1;
 }
 
 // the controller and, unless the call is done, the next attempt's set-up
 __device__ void controller_on(DevState* st, StageCoef* sc, double* __restrict__ hist,
                               const double* __restrict__ fixed) {
-  controller_core(st, hist);
+  const float eps = __uint_as_float(st->err_bits);
+  st->err_bits = 0;
+  st->ticket = 0;
+  step_apply(st, step_decide(*st, eps), eps, hist);
   if (!st->done) prepare_attempt(st, sc, fixed);
 }
 
