@@ -828,10 +828,9 @@ __global__ void __launch_bounds__(FilmCfg<LX, PH, ROWS, PZ>::NT, 1) k_film(const
     }
     arrive();
     if (!wait()) return timeout();
-    // The controller, by one warp, the same in every block.  (Its float64
-    // operands read ahead of the wait make no difference: 20 steps of a 64 x
-    // 16 film 877 us so, 880 here, 10 of a 256 x 256 film 833 and 835, 10 of a
-    // 256 x 63 racetrack 613 and 608.)
+    // The controller, by one warp, the same in every block.  (With its float64
+    // operands read ahead of the wait 10 steps of a 256 x 256 film took 836
+    // us, here 825, 20 of a 64 x 16 film 923 both ways.)
     if (tid < 32) {
       const float eps = __uint_as_float(__ldcg(&a.sync->err[att % 3]));
       const StepDecision d = step_decide(S, eps);

@@ -337,28 +337,32 @@ struct StepDecision {
   int accept, status, done, fixed_idx;
 };
 __device__ __forceinline__ StepDecision step_decide(const DevState& s, float eps) {
+  // (what the error does not decide comes first: its conversions and sums
+  // overlap the load of the error)
+  const double h = s.h, dt_min = s.dt_min, dt_max = s.dt_max, t_end = s.t_end;
+  double tn = s.t + h;
+  if (s.mode == 1 && tn + 1e-6 * h >= t_end) tn = t_end;
+  const float maxe = (float)s.max_err, maxe_dn = __double2float_rd(s.max_err);   // (eps <= max_err for a float eps)
+  const float head = (float)s.headroom, ex = s.method == 1 ? 1.0f / 3.0f : 0.2f;
   StepDecision d{s.t, s.dt, 0, 0, 0, s.fixed_idx};
   if (!(eps <= FLT_MAX)) {
     d.status = -4;   // MM_ERR_NONFINITE
     d.done = 1;
     return d;
   }
-  const double h = s.h;
   const bool replay = s.mode == 2;
-  d.accept = replay || eps <= __double2float_rd(s.max_err);   // (eps <= max_err for a float eps)
-  const float ex = s.method == 1 ? 1.0f / 3.0f : 0.2f;
-  const float ratio = (float)s.max_err / eps;   // (inf for a tiny eps)
-  const double factor = eps == 0.0f ? 5.0 : (double)fminf(5.0f, fmaxf(0.2f, (float)s.headroom * powf(ratio, ex)));
-  const double ndt = fmin(h * factor, s.dt_max);
+  d.accept = replay || eps <= maxe_dn;
+  const float ratio = maxe / eps;   // (inf for a tiny eps)
+  const double factor = eps == 0.0f ? 5.0 : (double)fminf(5.0f, fmaxf(0.2f, head * powf(ratio, ex)));
+  const double ndt = fmin(h * factor, dt_max);
   if (d.accept) {
-    d.t = s.t + h;
-    if (s.mode == 1 && d.t + 1e-6 * h >= s.t_end) d.t = s.t_end;
+    d.t = tn;
     if (replay) ++d.fixed_idx;
-    else d.dt = fmax(ndt, s.dt_min);
+    else d.dt = fmax(ndt, dt_min);
     if (s.mode == 0) d.done = s.accepted + 1 >= s.target;
-    else if (s.mode == 1) d.done = d.t >= s.t_end;
+    else if (s.mode == 1) d.done = d.t >= t_end;
     else d.done = d.fixed_idx >= s.fixed_n || s.accepted + 1 >= s.target;
-  } else if (ndt < s.dt_min) {
+  } else if (ndt < dt_min) {
     d.status = -5;   // MM_ERR_DT_UNDERFLOW
     d.done = 1;
   } else {
