@@ -301,7 +301,10 @@ int mm_sync(mm_ctx* ctx);
  * programmatic-dependent-launch overlap; the earlier-stage sums, a branch
  * beside the (y, z) part in the graph, run in line here), so the sum can
  * exceed the graph's time per attempt.  L2 is not
- * flushed between launches.  MM_ERR_STATE before set_m and unless the context
+ * flushed between launches.  Films and stacks of two to four layers are
+ * measured with their stage kernels too, which mm_step runs on them only after
+ * mm_set_yz_kernels with 1 or 2: by default it runs one persistent kernel.
+ * MM_ERR_STATE before set_m and unless the context
  * steps with the fused row-stage kernels (RK45, exact demag, no periodic x
  * axis, no spin-transfer torque); the controller's errors as mm_step. */
 int mm_profile_attempts(mm_ctx* ctx, int attempts, int max, int* kinds, double* us, int* n_out);
@@ -320,11 +323,17 @@ int mm_profile_attempts(mm_ctx* ctx, int attempts, int max, int* kinds, double* 
  * 128, 256 or 512 (MM_ERR_ARG otherwise).  *active (may be NULL) receives the
  * kernels in use: 1 or 2, or 0 on a grid that has no choice (none of the
  * cluster kernel's planes: the general convolution, or on larger grids with
- * open axes, 32 <= py <= 1024 and 16 <= pz <= 128 the three kernels).  The
- * stepping graph is captured again at the next step.  Films (one layer of
- * more than 8 rows, y not periodic) step with a persistent kernel that holds
- * its own (y, z) part by default; with which = 1 or 2 they step with the
- * stage kernels. */
+ * open axes, 32 <= py <= 1024, 16 <= pz <= 128 and room for their buffers the
+ * three kernels).  The
+ * stepping graph is captured again at the next step.
+ * Films and stacks of two to four layers (more than 8 rows, y and z not
+ * periodic) step with a persistent kernel that holds its own (y, z) part by
+ * default; there *active names the kernels of the field getters and
+ * mm_demag_apply.  With which = 1 or 2 such a context steps with the stage
+ * kernels.  That is the better choice for four and more films of 256 x 256 or
+ * eight of 128 x 128 stepped at once from several threads: the persistent
+ * kernels take turns on the device (eight films of 256 x 256: 513 us per step
+ * of all, 374 us with the stage kernels; one alone 65 and 108). */
 int mm_set_yz_kernels(mm_ctx* ctx, int which, int* active);
 
 /* FP32 fused multiply-add throughput of `device` (no counterpart in the

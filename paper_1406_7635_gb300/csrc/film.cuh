@@ -1,15 +1,16 @@
-// Persistent RK kernel of 2-D films: whole Runge-Kutta attempts (Sec. IV) in
-// one cooperative launch.
+// Persistent RK kernel of 2-D films and stacks of two to four layers: whole
+// Runge-Kutta attempts (Sec. IV) in one cooperative launch.
 //
 // A film's attempt is a chain of small steps that cannot overlap (stage input,
 // x transform, y transform and kernel product, inverse x transform, field,
 // next stage input), so one kernel per step pays a launch, a cold start
 // (state, tables, codes, material tables) and a drain several times per
 // stage.  Here the blocks stay resident for as many attempts as the call
-// needs: block b owns ROWS film rows and CPB kx columns, keeps its m, its
-// stage torques, its codes and its columns' kernel octant in shared memory,
-// and exchanges only the spectrum (through L2) and the rows that the
-// neighbours' stencils read.  Per stage:
+// needs: block b owns ROWS film rows and CPB kx columns, keeps its codes,
+// couplings, material tables, stage input and (where they fit) its columns'
+// kernel octant in shared memory, its m and stage torques in global memory
+// (read back by the thread that wrote them), and exchanges only the spectrum
+// (through L2) and the rows that the neighbours' stencils read.  Per stage:
 //
 //   rows:     stage input -> x R2C of the block's rows -> spec1[c][kx][y]
 //   -- grid barrier --
@@ -18,21 +19,28 @@
 //   -- grid barrier --
 //   rows:     x C2R -> B_demag -> field, torque k_s -> next stage input
 //
-// and after the last stage one more barrier for the maximum step error; the
-// controller then runs redundantly in every block (same inputs, same
-// result), block 0 keeps the device state.  Both spectrum exchanges write
-// scattered (8 ROWS or 8 CPB bytes) and read contiguous runs.
+// and after the last stage one more barrier for the maximum step error (13
+// per RK45 attempt); the controller then runs redundantly in every block
+// (same inputs, same result), block 0 keeps the device state.  Both spectrum
+// exchanges write scattered (8 ROWS or 8 CPB bytes) and read contiguous runs.
 //
-// Bound by latency: a stage is two grid barriers (about 1.4 us each with the
-// write-out before them) and, on every block, a serial chain of short
-// transforms; bandwidth and arithmetic are far from their limits.  What the
-// design buys is that chain without launches and cold starts.  Measured, us
-// per RK45 step, stage kernels in a graph -> this kernel: 64 x 16 film 83 ->
-// 38, 128 x 128 99 -> 46, 256 x 256 130 -> 64, 500 x 387 353 -> 175; 256 x 63
-// periodic with a Zhang-Li torque 141 -> 55 (RK23 73 -> 29).  On the way, for
-// 256 x 256: block-wide transform passes 118, 16 values per lane 78, 8 values
-// per lane with the material tables in shared memory and the earlier-stage
-// sums computed while the barrier waits 64.
+// Bound by latency: a stage is two grid barriers and, on every block, a serial
+// chain of short transforms; bandwidth and arithmetic are far from their
+// limits.  Share of a step that a block spends at the barriers / in the column
+// phase / in the rows' transforms / in the cells, by clock stamps: 64 x 16 film
+// (a block without rows) 67 / 16 / 3 / 4 %, 256 x 256 19 / 32 / 25 / 11 %, 500
+// x 387 7 / 48 / 26 / 10 %, 96 x 96 x 4 stack 18 / 37 / 23 / 8 % (a wait
+// includes the other blocks' work).  What the design buys is that chain without launches and cold
+// starts.  Measured, us per RK45 step, stage kernels in a graph -> this
+// kernel: 64 x 16 film 81 -> 37, 128 x 128 74 -> 44, 256 x 256 109 -> 65, 500
+// x 387 351 -> 174, 96 x 96 x 4 140 -> 64; 256 x 200 periodic 137 -> 56, with
+// RK23 and a Zhang-Li torque 73 -> 31.  A block holds most of a
+// multiprocessor's registers, so contexts stepped at once from several
+// threads take turns: eight films of 256 x 256 take 513 us per step of all,
+// 374 with the stage kernels (four: 257 and 212; eight of 500 x 387: 1388 and
+// 2162).  Fewer registers for more blocks per multiprocessor took eight 128 x
+// 128 films from 201 to 168 us (143 with the stage kernels) and slowed one
+// alone by 2 %.
 //
 // Every wait at a barrier is bounded; a wait that gives up records
 // MM_ERR_TIMEOUT, and m, t and dt stay those of the last accepted attempt

@@ -46,8 +46,8 @@ struct FilmPlan {
   size_t smem = 0;
 };
 // Plan of a fused grid of one to four layers with open y and z axes and more
-// than 8 cells along y, on the current device; false where the kernel does not apply (its blocks must all be
-// resident at once).  Sets the kernel's shared-memory limit.
+// than 8 cells along y, on the current device; false where the kernel does not
+// apply (its blocks must all be resident at once).  Sets the kernel's shared-memory limit.
 bool film_plan(const Geom& g, FilmPlan* plan);
 cudaError_t launch_film(const FilmPlan& plan, const FilmArgs& args, cudaStream_t s);
 

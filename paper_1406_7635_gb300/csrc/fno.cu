@@ -411,7 +411,8 @@ constexpr int kYSplit = 8;   // most row ranges of the tiled y product
 // column, jj, jj + JT, ..: one read of x serves them all and the reads of f
 // are the same in most of a warp.  With this and the same in k_yexpand_t a
 // 512 x 512 forward pass of width 32, 24 modes takes 537 us (556 at one output
-// per thread), the gradient of four such samples 4.17 ms (4.40).  Staging f by
+// per thread), the gradient of four such samples 4.17 ms (4.40)
+// with the copy of the gradient to the host, whose time varies by a millisecond.  Staging f by
 // asynchronous copies beside the reads of x, without a division per value, took
 // the forward pass from 484 to 462 us (with the 16-byte GEMM loads and the
 // packed layer kernel in place).
@@ -707,7 +708,8 @@ __global__ void __launch_bounds__(kPwNT) k_pointwise(int H, int W, int K2, const
 // instruction issue beside the FP32 units: two channels go in one packed
 // multiply-add, each rounded as a scalar one.  With this and z left out where
 // no gradient follows, a 512 x 512 forward pass of width 32, 24 modes takes
-// 484 us (512 before), the gradient of four samples 3.94 ms (4.2 to 4.8).
+// 484 us (512 before), the gradient of four samples 3.9 to 4.7 ms (4.2 to
+// 4.8; 0.6 to 1.4 ms of it the copy of the gradient to the host).
 __device__ __forceinline__ unsigned long long dup2(float a) {
   unsigned long long r;
   asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));

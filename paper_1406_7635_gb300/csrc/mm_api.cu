@@ -5,8 +5,9 @@
 // is captured once into a CUDA graph and replayed.  The controller runs on the
 // device and marks the call done; the host only replays the graph and reads the
 // device state back at a few check points, so steps are taken without a
-// host round trip per step.  Films run whole attempts in one persistent
-// kernel instead (film.cuh): one launch for all steps of a call.
+// host round trip per step.  Films and stacks of two to four layers run whole
+// attempts in one persistent kernel instead (film.cuh): one launch for the
+// first stage of a new state, one for up to kFilmAttempts attempts.
 #include <algorithm>
 #include <cmath>
 #include <cstdio>

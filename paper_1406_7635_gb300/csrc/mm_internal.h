@@ -120,7 +120,7 @@ struct DevState {
   int call_attempts;         // attempts since the last begin
   int precession;
   int method;               // 0 Dormand-Prince RK45, 1 Bogacki-Shampine RK23
-  long long wait_cycles;    // limit of a kernel's wait on its tensor copies (SM clock cycles)
+  long long wait_cycles;    // limit of a wait on tensor copies or at a film's grid barrier (SM clock cycles)
 };
 
 // default wait limit: 2^30 cycles, about half a second at the maximum SM clock
@@ -196,7 +196,9 @@ bool yz3_plan(const Geom& g);
 // Grids beyond the cluster kernel's planes (fused_plan refuses them) that the
 // three kernels can serve: marks g as fused without a residue split
 // (large_grid), so that the context steps with the row-stage kernels and
-// always convolves with the three kernels.
+// convolves with the three kernels.  A context asks for it once the general
+// convolution's buffers are in place and gives it up where there is no room
+// for the others.
 bool large_plan(Geom& g);
 // 2-D grids: y forward, kernel product and y inverse of a kx plane in one
 // block (fft_yz3.cu), in place in the spectrum; y2d_plan(g) tells whether
