@@ -360,9 +360,11 @@ int bfail(int code, const std::string& msg) {
 #define MMB_CUDA(call)                                                                        \
   do {                                                                                        \
     cudaError_t e_ = (call);                                                                  \
-    if (e_ != cudaSuccess)                                                                    \
+    if (e_ != cudaSuccess) {                                                                  \
+      (void)cudaGetLastError(); /* reported here, not by the next call's check */             \
       return bfail(e_ == cudaErrorMemoryAllocation ? MM_ERR_OOM : MM_ERR_CUDA,                \
                    std::string(#call) + ": " + cudaGetErrorString(e_));                       \
+    }                                                                                         \
   } while (0)
 
 BPtrs bptrs(const BClass& c) {

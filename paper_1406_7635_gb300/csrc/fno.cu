@@ -1374,9 +1374,11 @@ int ffail(int code, const std::string& msg) {
 #define MMF_CUDA(call)                                                                        \
   do {                                                                                        \
     cudaError_t e_ = (call);                                                                  \
-    if (e_ != cudaSuccess)                                                                    \
+    if (e_ != cudaSuccess) {                                                                  \
+      (void)cudaGetLastError(); /* reported here, not by the next call's check */             \
       return ffail(e_ == cudaErrorMemoryAllocation ? MM_ERR_OOM : MM_ERR_CUDA,                \
                    std::string(#call) + ": " + cudaGetErrorString(e_));                       \
+    }                                                                                         \
   } while (0)
 
 float* P_(mm_fno* f, int k) { return f->prm + f->off[k]; }

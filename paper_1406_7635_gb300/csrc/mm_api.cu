@@ -33,9 +33,11 @@ int fail(int code, const std::string& msg) {
 #define MM_CUDA(call)                                                                  \
   do {                                                                                 \
     cudaError_t e_ = (call);                                                           \
-    if (e_ != cudaSuccess)                                                             \
+    if (e_ != cudaSuccess) {                                                           \
+      (void)cudaGetLastError(); /* reported here, not by the next call's check */      \
       return fail(e_ == cudaErrorMemoryAllocation ? MM_ERR_OOM : MM_ERR_CUDA,          \
                   std::string(#call) + ": " + cudaGetErrorString(e_));                 \
+    }                                                                                  \
   } while (0)
 
 constexpr double kPi = 3.14159265358979323846;
@@ -252,6 +254,7 @@ int apply_yz_choice(mm_ctx* c) {
   if (want && !c->yzt) {
     cudaError_t e = cudaMalloc((void**)&c->yzt, yz3_bytes(c->g));
     if (e != cudaSuccess) {
+      (void)cudaGetLastError();
       c->yzt = nullptr;
       return fail(e == cudaErrorMemoryAllocation ? MM_ERR_OOM : MM_ERR_CUDA,
                   std::string("(y, z) buffer: ") + cudaGetErrorString(e));
@@ -1156,10 +1159,7 @@ int mm_set_pbc(mm_ctx* c, int px, int py, int pz) {
   if (e == cudaSuccess) {
     prepare_large(c);
     const int rc = apply_yz_choice(c);
-    if (rc) {
-      (void)cudaGetLastError();
-      return rc;
-    }
+    if (rc) return rc;
     // one convolution outside any capture (launch attributes), as at creation
     Buffers nb = b;
     nb.st = nullptr;
@@ -1512,7 +1512,10 @@ int mm_surrogate_train(mm_ctx* c, mm_fno* net, double ms_ref, int n_pairs, int t
     c->k1_valid = false;
     return code;
   };
-  if (e != cudaSuccess) return done(fail(MM_ERR_OOM, "no room for the training pairs"));
+  if (e != cudaSuccess) {
+    (void)cudaGetLastError();   // (the state is put back by calls that check it)
+    return done(fail(MM_ERR_OOM, "no room for the training pairs"));
+  }
   unsigned long long st = seed * 0x9E3779B97F4A7C15ULL + 7;
   auto unif = [&]() {   // splitmix64 -> (0, 1)
     st += 0x9E3779B97F4A7C15ULL;
@@ -1563,6 +1566,7 @@ int mm_surrogate_train(mm_ctx* c, mm_fno* net, double ms_ref, int n_pairs, int t
   e = cudaMalloc((void**)&ub, (size_t)batch * n3 * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc((void**)&yb, (size_t)batch * n3 * sizeof(float));
   if (e != cudaSuccess) {
+    (void)cudaGetLastError();
     cudaFree(ub);
     cudaFree(yb);
     return done(fail(MM_ERR_OOM, "no room for the training batch"));

@@ -280,3 +280,45 @@ def test_a_longer_replay_sequence_without_room_keeps_the_one_there(fake):
     assert fake.rt.fake_used() == held + 8 * 996
     ctx.close()
     assert fake.rt.fake_used() == base
+
+
+def test_no_room_in_a_call_is_no_error_of_the_next(fake):
+    """Calls that allocate on the way: the (y, z) buffer asked for, the table
+    of the spin torques, the surrogate's accumulators and its training pairs.
+    Each reports MM_ERR_OOM and the context steps on; training puts m back."""
+    ctx = context(fake, (32, 32, 16))
+    ctx.set_yz_kernels(1)
+    net = fake.FNO(16, 40, width=8, layers=1, modes_x=4, modes_y=4, max_batch=2)
+    film = context(fake, (40, 16, 1))
+    film.set_material(0, 8e5, 1.3e-11, 0.1, jcur=(1e12, 0.0, 0.0), xi=0.05)
+    film.step(1)
+    m = film.get_m()
+
+    def torque():
+        film.enable_stt(True, False)
+        film.step(1)
+
+    calls = [(lambda: ctx.set_yz_kernels(2), ctx), (torque, film),
+             (lambda: film.set_demag_surrogate(net, 8e5), film),
+             (lambda: film.train_surrogate(net, 8e5, 2, 1, 0, 0.0, 1, 1, 1e-3), film)]
+    for call, c in calls:
+        for k in range(6):
+            fake.rt.fake_fail_at(k)
+            try:
+                call()
+            except fake.MMError as e:
+                assert e.code == MM_ERR_OOM
+            else:
+                break
+            fake.rt.fake_fail_at(-1)
+            assert np.array_equal(film.get_m(), m)
+            ctx.step(1)
+            ctx.get_bdemag()
+            film.set_m(m)
+        else:
+            raise AssertionError("more allocations than expected")
+        fake.rt.fake_fail_at(-1)
+        assert k > 0
+        film.set_demag_surrogate(None, 8e5)
+    for c in (ctx, film, net):
+        c.close()
